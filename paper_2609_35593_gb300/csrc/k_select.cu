@@ -279,6 +279,16 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   return y;
 }
 
+// a / b for b in [2^-54, 2^4] (here a product of factors clamped at eps = 1e-4): one SFU
+// reciprocal and a multiplication.  __fdividef gives the same bits there (compared on 1e9
+// random pairs, denormal numerators included) but spends further instructions on
+// denominators outside that range.
+__device__ __forceinline__ float div_fast(float a, float b) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+  return a * r;
+}
+
 // Order-preserving map of a float to uint32; every non-NaN value maps above 0, so 0 can
 // mark "not a candidate".  -0 is folded onto +0; NaN maps to the lowest candidate value.
 __device__ __forceinline__ uint32_t order_key(float x) {
@@ -290,21 +300,19 @@ __device__ __forceinline__ uint32_t order_key(float x) {
 
 // ------------------------------------------------------------------------------------
 // Exact top-m for one warp over keys kk[0..n) in shared memory (block j has key kk[j]):
-// the m largest keys, ties to the lower block index (the order the oracle uses).  With
-// `member` set, only blocks whose bit in member[] equals `want` take part.  Result: the
-// chosen blocks' bits in sel[words] (cleared first).
+// the m largest keys, ties to the lower block index (the order the oracle uses).  Result:
+// the chosen blocks' bits in sel[words].
 //
 // 1. lower bound: the m-th largest value among every lane's local top-ceil(m/32) keys is
 //    <= the m-th largest key overall (those 32 ceil(m/32) values include m entries);
-// 2. survivors: the participating keys >= that bound (usually about 1.5 m of them) are
-//    compacted, in block order, into a short list;
+// 2. survivors: the keys >= that bound (usually about 1.5 m of them) are compacted, in block
+//    order, into a short list;
 // 3. the m-th largest survivor T is found by a radix select over the survivors (8-bit
-//    digits; select_radix), or bit by bit without radix counters (select_exact), and the
-//    survivors > T plus the lowest-index ones == T are chosen.
-// When m needs more than kTopK candidates per lane, or too many keys tie at the bound,
-// step 3 runs bit by bit on all participating keys instead (same result, slower).  The
-// restoration rounds use warp_topm_pair below, which selects on both sides of the drop set
-// at once.
+//    digits; select_radix) and the survivors > T plus the lowest-index ones == T are chosen.
+// When m needs more than kTopK candidates per lane, warp_topm_large selects on all keys; when
+// too many keys tie at the bound, step 3 runs bit by bit on all keys (select_exact: same
+// result, slower).  The restoration rounds use warp_topm_pair (m <= 64) or warp_topm_large,
+// which select on both sides of the drop set at once.
 // ------------------------------------------------------------------------------------
 constexpr int kTopK = 4;          // lane-local candidates: fast path for m <= 128
 constexpr int kSurvivors = 256;   // capacity of the survivor list
@@ -488,18 +496,159 @@ __device__ void select_radix(const uint32_t* keys, const uint16_t* idx, int n, i
   }
 }
 
+// Exact selection for large m, by a radix select over all n keys whose counters live in the
+// survivor scratch (256 words, two 16-bit counters each: 256 digits of each side).  PAIR: the m
+// largest keys among the blocks of the drop set Dw into selD and the m largest among the
+// other candidates into selB at once (every key belongs to one side, so both sides share each
+// pass); otherwise the m largest of all keys into selD.  Ties go to the lower index; a side
+// with fewer than m blocks is taken whole.  Three passes over the keys, 32 consecutive blocks
+// at a time so that a mask word is one ballot: counts by the top byte, counts by the second
+// byte of the keys that share the m-th key's top byte, then the choice; the few keys that
+// share its upper 16 bits are ranked among themselves (a side with more than 128 of those,
+// heavy ties, takes select_exact).  A bit-by-bit search over the keys, which this replaces
+// for m > 64 (rounds) and m > 128 (initial selection), makes up to 32 passes per side: at 64
+// views and half the blocks dropped (m = 171, 1369 keys) the round kernel took 774 us with it
+// and 313 us with this.
+template <bool PAIR>
+__device__ void warp_topm_large(const uint32_t* kk, int n, int m, const uint32_t* Dw,
+                                uint32_t* selD, uint32_t* selB, int words, uint32_t* sk,
+                                uint16_t* si) {
+  constexpr int kSides = PAIR ? 2 : 1;
+  constexpr int kHalf = kSurvivors / 2;
+  const int lane = threadIdx.x & 31;
+  const uint32_t below = (1u << lane) - 1u;
+  int prefix[2] = {0, 0}, need[2] = {m, m}, cnt[2] = {0, 0};
+#pragma unroll
+  for (int pass = 0; pass < 2; ++pass) {
+    reinterpret_cast<uint4*>(sk)[lane] = make_uint4(0u, 0u, 0u, 0u);
+    if (PAIR) reinterpret_cast<uint4*>(sk)[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    __syncwarp();
+#pragma unroll 4
+    for (int w = 0; w < words; ++w) {
+      const int x = 32 * w + lane;
+      if (x < n) {
+        const uint32_t v = kk[x];
+        const int side = PAIR ? (int)(~(Dw[w] >> lane) & 1u) : 0;  // 0: in D (or all), 1: not
+        const uint32_t d = pass == 0 ? v >> 24 : (v >> 16) & 255u;
+        if (pass == 0 || (int)(v >> 24) == (side ? prefix[1] : prefix[0]))
+          atomicAdd(&sk[128 * side + (d >> 1)], 1u << (16 * (d & 1u)));
+      }
+    }
+    __syncwarp();
+    // lane l owns digits base + 7 .. base, base = 8 (31 - l): lane 0 the highest; one scan
+    // carries both sides' counts (16 bits each; n <= 4096)
+    uint32_t c[2][4];
+    int sum = 0;
+#pragma unroll
+    for (int t = 0; t < kSides; ++t) {
+      const uint4 q = reinterpret_cast<const uint4*>(sk)[32 * t + 31 - lane];
+      c[t][0] = q.w; c[t][1] = q.z; c[t][2] = q.y; c[t][3] = q.x;
+      const uint32_t two = (q.x + q.y) + (q.z + q.w);  // no carry: at most 4096 in all
+      sum += (int)((two & 0xffffu) + (two >> 16)) << (16 * t);
+    }
+    int inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += y;
+    }
+    const int total = __shfl_sync(kFull, inc, 31);
+#pragma unroll
+    for (int t = 0; t < kSides; ++t) {
+      if (pass == 0) need[t] = min(need[t], (total >> (16 * t)) & 0xffff);
+      const int mine = (sum >> (16 * t)) & 0xffff;
+      const int in_t = (inc >> (16 * t)) & 0xffff, ex_t = in_t - mine;
+      const uint32_t who = __ballot_sync(kFull, ex_t < need[t] && need[t] <= in_t);
+      int found = 0;  // digit | count << 8 | keys above the digit << 20
+      if ((who >> lane) & 1u) {
+        int run = ex_t;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int k = (int)((i & 1) ? c[t][i >> 1] & 0xffffu : c[t][i >> 1] >> 16);
+          if (found == 0 && run + k >= need[t]) found = (8 * (31 - lane) + 7 - i) | (k << 8);
+          if (found == 0) run += k;
+        }
+        need[t] -= run;
+      }
+      const int src = who ? __ffs(who) - 1 : 0;  // none: need is 0, nothing to choose
+      found = __shfl_sync(kFull, found, src);
+      need[t] = __shfl_sync(kFull, need[t], src);
+      prefix[t] = (prefix[t] << 8) | (found & 255);
+      cnt[t] = found >> 8;
+      if (!who) prefix[t] = pass == 0 ? 255 : 0xffff;
+    }
+    __syncwarp();
+  }
+  // keys above gt[side] are chosen; those whose upper half is eq[side] are listed
+  int gt[2], eq[2], listed[2] = {0, 0};
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const bool all = cnt[t] == need[t] && need[t] > 0;
+    gt[t] = all ? prefix[t] - 1 : prefix[t];
+    eq[t] = (all || need[t] == 0) ? -2 : prefix[t];
+  }
+#pragma unroll 2
+  for (int w = 0; w < words; ++w) {
+    const int x = 32 * w + lane;
+    const uint32_t v = x < n ? kk[x] : 0u;
+    const uint32_t dw = PAIR ? Dw[w] : kFull;
+    const bool inD = (dw >> lane) & 1u;
+    const int v16 = (int)(v >> 16);
+    const uint32_t pick = __ballot_sync(kFull, x < n && v16 > (PAIR && !inD ? gt[1] : gt[0]));
+    const uint32_t tie = __ballot_sync(kFull, x < n && v16 == (PAIR && !inD ? eq[1] : eq[0]));
+    if (lane == 0) {
+      selD[w] = pick & dw;
+      if (PAIR) selB[w] = pick & ~dw;
+    }
+    if (tie) {
+      const uint32_t tD = tie & dw, tB = tie & ~dw;
+      const int t = inD ? 0 : 1;
+      const int pos = (inD ? listed[0] : listed[1]) + __popc((inD ? tD : tB) & below);
+      if (((tie >> lane) & 1u) && pos < kHalf) {
+        sk[kHalf * t + pos] = v;
+        si[kHalf * t + pos] = (uint16_t)x;
+      }
+      listed[0] += __popc(tD);
+      listed[1] += __popc(tB);
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int t = 0; t < kSides; ++t) {
+    if (eq[t] < 0) continue;
+    uint32_t* sel = t ? selB : selD;
+    const int L = listed[t];
+    if (L > kHalf) {
+      select_exact(kk, nullptr, n, m, PAIR ? Dw : nullptr, t == 0, sel);
+      continue;
+    }
+    for (int x = lane; x < L; x += 32) {  // the list is in ascending block order
+      const uint32_t v = sk[kHalf * t + x];
+      int rank = 0;
+      for (int o = 0; o < L; ++o) {
+        const uint32_t u = sk[kHalf * t + o];
+        rank += (u > v || (u == v && o < x)) ? 1 : 0;
+      }
+      if (rank < need[t]) {
+        const int j = si[kHalf * t + x];
+        atomicOr(&sel[j >> 5], 1u << (j & 31));
+      }
+    }
+  }
+  __syncwarp();
+}
+
 // The lower bound of step 1 with KT = ceil(m / 32) keys kept per lane: the m-th largest of
-// the lanes' KT largest participating keys.
+// the lanes' KT largest keys.
 template <int KT>
-__device__ __forceinline__ uint32_t lane_topk_bound(const uint32_t* kk, int n, int m,
-                                                    const uint32_t* member, bool want) {
+__device__ __forceinline__ uint32_t lane_topk_bound(const uint32_t* kk, int n, int m) {
   const int lane = threadIdx.x & 31;
   uint32_t top[KT];
 #pragma unroll
   for (int k = 0; k < KT; ++k) top[k] = 0u;
 #pragma unroll 2
   for (int x = lane; x < n; x += 32) {
-    uint32_t v = takes_part(member, want, x) ? kk[x] : 0u;
+    uint32_t v = kk[x];
 #pragma unroll
     for (int k = 0; k < KT; ++k) {
       const uint32_t hi = max(top[k], v);
@@ -510,34 +659,33 @@ __device__ __forceinline__ uint32_t lane_topk_bound(const uint32_t* kk, int n, i
   return mth_largest(top, m);
 }
 
-// Requires m <= number of participating blocks.  sk/si: survivor scratch (kSurvivors);
-// hist: 256 words for select_radix on the survivors (NULL: bit-by-bit select_exact).
+// Requires m <= n.  sk/si: survivor scratch (kSurvivors); hist: 256 words for select_radix on
+// the survivors.
+// LARGE: m may exceed 32 kTopK.
+template <bool LARGE>
 __device__ void warp_topm(const uint32_t* kk, int n, int m, uint32_t* sel, int words,
-                          uint32_t* sk, uint16_t* si, const uint32_t* member = nullptr,
-                          bool want = true, uint32_t* hist = nullptr) {
+                          uint32_t* sk, uint16_t* si, uint32_t* hist) {
   const int lane = threadIdx.x & 31;
+  if (LARGE && m > 32 * kTopK) {
+    warp_topm_large<false>(kk, n, m, nullptr, sel, nullptr, words, sk, si);
+    return;
+  }
   for (int w = lane; w < words; w += 32) sel[w] = 0u;
   __syncwarp();
   if (m <= 0) return;
-  const int K = (m + 31) / 32;
-  if (K > kTopK) {
-    select_exact(kk, nullptr, n, m, member, want, sel);
-    __syncwarp();
-    return;
-  }
-  // 1. lane-local top-K (descending) of the participating keys, then the lower bound
+  // 1. lane-local top-K (descending), then the lower bound
   uint32_t bound;
-  switch (K) {
-    case 1: bound = lane_topk_bound<1>(kk, n, m, member, want); break;
-    case 2: bound = lane_topk_bound<2>(kk, n, m, member, want); break;
-    case 3: bound = lane_topk_bound<3>(kk, n, m, member, want); break;
-    default: bound = lane_topk_bound<4>(kk, n, m, member, want); break;
+  switch ((m + 31) / 32) {
+    case 1: bound = lane_topk_bound<1>(kk, n, m); break;
+    case 2: bound = lane_topk_bound<2>(kk, n, m); break;
+    case 3: bound = lane_topk_bound<3>(kk, n, m); break;
+    default: bound = lane_topk_bound<4>(kk, n, m); break;
   }
-  // 2. survivors (participating, >= bound), compacted in block order
+  // 2. survivors (>= bound), compacted in block order
   int cnt = 0;
   for (int x0 = 0; x0 < n; x0 += 32) {
     const int x = x0 + lane;
-    const bool keep = x < n && kk[x] >= bound && takes_part(member, want, x);
+    const bool keep = x < n && kk[x] >= bound;
     const uint32_t b = __ballot_sync(kFull, keep);
     const int pos = cnt + __popc(b & ((1u << lane) - 1u));
     if (keep && pos < kSurvivors) {
@@ -547,13 +695,11 @@ __device__ void warp_topm(const uint32_t* kk, int n, int m, uint32_t* sel, int w
     cnt += __popc(b);
   }
   __syncwarp();
-  // 3. exact selection on the survivors (or on every participating key if they overflowed)
+  // 3. exact selection on the survivors (or on every key if they overflowed)
   if (cnt > kSurvivors)
-    select_exact(kk, nullptr, n, m, member, want, sel);
-  else if (hist)
-    select_radix(sk, si, cnt, m, hist, sel);
+    select_exact(kk, nullptr, n, m, nullptr, true, sel);
   else
-    select_exact(sk, si, cnt, m, nullptr, true, sel);
+    select_radix(sk, si, cnt, m, hist, sel);
   __syncwarp();
 }
 
@@ -561,10 +707,11 @@ __device__ void warp_topm(const uint32_t* kk, int n, int m, uint32_t* sel, int w
 struct LaneTop2 {
   uint32_t d1 = 0, d2 = 0, b1 = 0, b2 = 0;  // in D: largest, second; outside D: same
   __device__ __forceinline__ void add(uint32_t v, bool inD) {
-    uint32_t& a1 = inD ? d1 : b1;
-    uint32_t& a2 = inD ? d2 : b2;
-    a2 = max(a2, min(a1, v));
-    a1 = max(a1, v);
+    const uint32_t vd = inD ? v : 0u, vb = inD ? 0u : v;
+    d2 = max(d2, min(d1, vd));
+    d1 = max(d1, vd);
+    b2 = max(b2, min(b1, vb));
+    b1 = max(b1, vb);
   }
 };
 
@@ -607,7 +754,11 @@ __device__ __forceinline__ uint32_t mth_of_64(uint32_t a, uint32_t b, int m) {
 // positions); each side then selects exactly (radix select on its survivors).
 // Returns true when the chosen blocks went to lst (restores at lst[0..m), drops at
 // lst[m..2m) with bit 15 set) instead of the bitmasks; lst lies in the key area after its
-// first 256 words (the radix counters).
+// first 256 words (the radix counters).  Above m = 32 the bound is loose (the m-th of only 64
+// values) and the survivors often overflow their 128 places per side; LARGE kernels then select
+// on all keys with warp_topm_large (m = 53 over 2142 keys at 100 views: 1611 us for the round
+// with the bit-by-bit search, 724 us with it).
+template <bool LARGE>
 __device__ bool warp_topm_pair(const uint32_t* kk, int n, int m, const uint32_t* Dw,
                                const LaneTop2& top, uint32_t* selD, uint32_t* selB,
                                int words, uint32_t* sk, uint16_t* si, uint16_t* lst) {
@@ -678,6 +829,10 @@ __device__ bool warp_topm_pair(const uint32_t* kk, int n, int m, const uint32_t*
     __syncwarp();
     return true;
   }
+  if (LARGE) {
+    warp_topm_large<true>(kk, n, m, Dw, selD, selB, words, sk, si);
+    return false;
+  }
   if (cntD > kHalf)
     select_exact(kk, nullptr, n, m, Dw, true, selD);
   else
@@ -711,14 +866,78 @@ __device__ __forceinline__ uint32_t valid_bits(int w, int n) {
   return rem >= 32 ? kFull : (rem <= 0 ? 0u : ((1u << rem) - 1u));
 }
 
+// g~ += sum_e P_j (z~_j - y~_i) and K += sum_e P_j over a list of n blocks, in list order, by
+// one warp (lane owns channels 2 lane, 2 lane + 1).  The list (shared memory, 16-byte
+// aligned) holds u16 entries j | flag; a flagged entry (bit 15) is subtracted.  Bound by
+// instruction issue and by the latency of the z~ rows (256 bytes each, from L2).  The weights
+// of 64 entries at a time are gathered by two loads of the warp and staged in wst (64
+// floats of shared memory) while the first rows are under way; eight rows are in flight
+// together, and a batch of eight costs one shared-memory load for its entries and two for
+// its weights instead of two loads per entry (k_score_rows at 64 views, 687 kept blocks a
+// row: 443 -> 408 us against weights handed round by shuffles, 492 with both loads).
+__device__ __forceinline__ void drift_sum(const uint16_t* lst, int n,
+                                          const float* __restrict__ Prow,
+                                          const float* __restrict__ zt, float y0, float y1,
+                                          float* wst, float& g0, float& g1, float& K) {
+  const int lane = threadIdx.x & 31;
+  const char* zl = reinterpret_cast<const char*>(zt + 2 * lane);
+  for (int c0 = 0; c0 < n; c0 += 64) {
+    float pw[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = c0 + 32 * u + lane;
+      pw[u] = 0.f;
+      if (e < n) {
+        const uint32_t v = lst[e];
+        pw[u] = __uint_as_float(__float_as_uint(Prow[v & 0x7fffu]) ^ ((v & 0x8000u) << 16));
+      }
+    }
+    const int cnt = min(64, n - c0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < cnt; k0 += 8) {
+      const uint4 ent = *reinterpret_cast<const uint4*>(lst + c0 + k0);
+      const uint32_t e2[4] = {ent.x, ent.y, ent.z, ent.w};
+      const bool full = k0 + 8 <= cnt;
+      float2 z[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t off = ((u & 1) ? e2[u >> 1] >> 16 : e2[u >> 1]) & 0x7fffu;
+        if (full || k0 + u < cnt) z[u] = *reinterpret_cast<const float2*>(zl + 256u * off);
+      }
+      if (k0 == 0) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) wst[32 * u + lane] = pw[u];
+        __syncwarp();
+      }
+#pragma unroll
+      for (int half = 0; half < 8; half += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(wst + k0 + half);
+        const float pj[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (full || k0 + half + u < cnt) {
+            // both channels in packed instructions (z - y as an exact fma with 1, so the
+            // bits are those of the scalar form)
+            float d0, d1;
+            ptx::fma2(d0, d1, z[half + u].x, z[half + u].y, 1.0f, 1.0f, -y0, -y1);
+            ptx::fma2(g0, g1, pj[u], pj[u], d0, d1, g0, g1);
+            K += pj[u];
+          }
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // g~ = sum_{j not in D} P_ij (z~_j - y~_i) and K = sum_{j not in D} P_ij for one row, by
 // one warp (lane owns channels 2*lane, 2*lane+1), in ascending j.  The kept blocks are
-// first compacted into idx[] (per-warp shared memory, >= nb entries) so that the loads of
-// eight blocks are in flight together.
+// first compacted into idx[] (per-warp shared memory, >= nb entries).
 __device__ __forceinline__ void kept_drift(const uint32_t* D, const SelPtrs& p,
                                            const float* __restrict__ Prow,
                                            const float* __restrict__ zt, float y0, float y1,
-                                           uint32_t* idx, float& g0, float& g1, float& K) {
+                                           uint16_t* idx, float* wst, float& g0, float& g1,
+                                           float& K) {
   const int lane = threadIdx.x & 31;
   // lane l compacts mask word w0 + l: one warp scan of the words' kept counts gives each
   // word's first list position, then each lane writes its own word's blocks (ascending)
@@ -733,70 +952,13 @@ __device__ __forceinline__ void kept_drift(const uint32_t* D, const SelPtrs& p,
       const int y = __shfl_up_sync(kFull, inc, o);
       if (lane >= o) inc += y;
     }
-    for (int pos = n + inc - c; keep; keep &= keep - 1u, ++pos) idx[pos] = w * 32 + __ffs(keep) - 1;
+    for (int pos = n + inc - c; keep; keep &= keep - 1u, ++pos) 
+      idx[pos] = (uint16_t)(w * 32 + __ffs(keep) - 1);
     n += __shfl_sync(kFull, inc, 31);
   }
   __syncwarp();
   g0 = g1 = K = 0.f;
-  for (int k0 = 0; k0 < n; k0 += 8) {
-    float pj[8];
-    float2 z[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (k0 + u < n) {
-        const int j = idx[k0 + u];
-        pj[u] = Prow[j];
-        z[u] = *reinterpret_cast<const float2*>(zt + (int64_t)j * 64 + 2 * lane);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (k0 + u < n) {
-        // g += P_j (z~_j - y~), both channels in packed instructions (z - y as an exact
-        // fma with 1, so the bits are those of the scalar form)
-        float d0, d1;
-        ptx::fma2(d0, d1, z[u].x, z[u].y, 1.0f, 1.0f, -y0, -y1);
-        ptx::fma2(g0, g1, pj[u], pj[u], d0, d1, g0, g1);
-        K += pj[u];
-      }
-    }
-  }
-  __syncwarp();
-}
-
-// The state after a round from the one before it: the restored blocks R join the kept set
-// and the dropped blocks X leave it, so g~ += sum_R P_k (z~_k - y~) - sum_X P_k (z~_k - y~)
-// and K += sum_R P_k - sum_X P_k over the 2m swapped blocks (exactly the kept-set sums of
-// Eq. 10-11 in exact arithmetic), taken in the order of their list (j | 0x8000 for a
-// dropped block).  Same lane layout and staging as kept_drift.
-__device__ __forceinline__ void swap_drift_list(const uint16_t* lst, int n,
-                                                const float* __restrict__ Prow,
-                                                const float* __restrict__ zt, float y0, float y1,
-                                                float& g0, float& g1, float& K) {
-  const int lane = threadIdx.x & 31;
-  for (int k0 = 0; k0 < n; k0 += 8) {
-    float pj[8];
-    float2 z[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      pj[u] = 0.f;
-      z[u] = make_float2(y0, y1);
-      if (k0 + u < n) {
-        const uint32_t e = lst[k0 + u];
-        const int j = (int)(e & 0x7fffu);
-        const float pv = Prow[j];
-        pj[u] = (e >> 15) ? -pv : pv;
-        z[u] = *reinterpret_cast<const float2*>(zt + (int64_t)j * 64 + 2 * lane);
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      g0 = fmaf(pj[u], z[u].x - y0, g0);
-      g1 = fmaf(pj[u], z[u].y - y1, g1);
-      K += pj[u];
-    }
-  }
-  __syncwarp();
+  drift_sum(idx, n, Prow, zt, y0, y1, wst, g0, g1, K);
 }
 
 // Per-warp scratch of the per-row kernels: keys [key_words(ld)] u32, survivor keys
@@ -827,7 +989,7 @@ __device__ __forceinline__ float delta_J(float G, float K, float dG, float u) {
   const float Kc = fmaxf(K, kEps), K2c = fmaxf(K + u, kEps);
   const float KK = Kc * Kc;
   const float num = fmaf(G * (K2c - Kc), K2c + Kc, -dG * KK);
-  return __fdividef(num, KK * (K2c * K2c));
+  return div_fast(num, KK * (K2c * K2c));
 }
 
 
@@ -838,17 +1000,24 @@ __device__ __forceinline__ float delta_J(float G, float K, float dG, float u) {
 constexpr int kRowWarps = 4;
 
 // Candidate keys of one row, four blocks per lane and load (rows are 16-byte aligned and
-// padded to a multiple of 32 entries).
-template <typename KeyFn>
-__device__ __forceinline__ void row_keys(int n, uint32_t* kk, KeyFn key_of) {
+// padded to a multiple of 32 entries; so is kk).  Keys past n are 0, below every candidate's.
+// Not unrolled: the row kernels wait on instruction fetch (2.4 of 13 stall cycles per issue
+// in the round kernel), and two quads per step made the rounds of the 32-view layer slower
+// (66.7 / 51.1 / 45.5 us against 62.9 / 47.7 / 43.3).
+template <typename KeyFn, typename SeenFn>
+__device__ __forceinline__ void row_keys(int n, uint32_t* kk, KeyFn key_of, SeenFn seen) {
   const int lane = threadIdx.x & 31;
-#pragma unroll 2
+#pragma unroll 1
   for (int j4 = 4 * lane; j4 < n; j4 += 128) {
     uint32_t k4[4];
     key_of(j4, k4);
+    if (j4 + 4 > n) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (j4 + u < n) kk[j4 + u] = k4[u];
+      for (int u = 1; u < 4; ++u)
+        if (j4 + u >= n) k4[u] = 0u;
+    }
+    seen(j4, k4);
+    *reinterpret_cast<uint4*>(kk + j4) = make_uint4(k4[0], k4[1], k4[2], k4[3]);
   }
   __syncwarp();
 }
@@ -924,8 +1093,10 @@ __device__ void cdf_extend(const uint32_t* kk, const float* __restrict__ Prow, u
 // 24 bits of SplitMix64 at seed + (h 4096 + i) 4096 + j; the full sign flip keeps the
 // smallest keys (complemented keys, ties still to the lower index).
 // KEY: the key variant (v.key), a template parameter so that the per-block key has no branch.
-template <int KEY>
-__global__ void __launch_bounds__(32 * kRowWarps, 9) k_score_rows(SelPtrs p, Budgets bud,
+// LARGE: some head's budget exceeds 32 kTopK (the selection on all keys is compiled in; it
+// takes more registers, and rows that long leave room for fewer warps anyway).
+template <int KEY, bool LARGE>
+__global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(SelPtrs p, Budgets bud,
                                                                   Variant v) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -951,7 +1122,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, 9) k_score_rows(SelPtrs p, Bud
     for (int u = 0; u < 4; ++u) {
       uint32_t key;
       if (KEY == 0)  // s_ij / max(1 - P_ij, eps), s_ij = P_ij sqrt(q_ij); the SFU's square root
-        key = order_key(__fdividef(pv[u] * sqrt_approx(qv[u]), fmaxf(1.0f - pv[u], kEps)));
+        key = order_key(div_fast(pv[u] * sqrt_approx(qv[u]), fmaxf(1.0f - pv[u], kEps)));
       else if (KEY == 1)
         key = order_key(pv[u]);
       else
@@ -959,8 +1130,8 @@ __global__ void __launch_bounds__(32 * kRowWarps, 9) k_score_rows(SelPtrs p, Bud
                                                  4096ull + (unsigned long long)(j + u)) >> 40) + 1u;
       k4[u] = (v.direction == 2) ? ~key : key;
     }
-  });
-  warp_topm(kk, p.ncand, bud.c[h], sel, p.words, sk, si, nullptr, true, hist);  // sel = kept
+  }, [](int, const uint32_t (&)[4]) {});
+  warp_topm<LARGE>(kk, p.ncand, bud.c[h], sel, p.words, sk, si, hist);  // sel = kept
   // drop set D0 = candidates not kept
   for (int w = lane; w < p.words; w += 32) sel[w] = valid_bits(w, p.ncand) & ~sel[w];
   __syncwarp();
@@ -977,7 +1148,8 @@ __global__ void __launch_bounds__(32 * kRowWarps, 9) k_score_rows(SelPtrs p, Bud
   __syncwarp();
   const float2 y = *reinterpret_cast<const float2*>(p.ytil + ri * 64 + 2 * lane);
   float g0, g1, K;
-  kept_drift(sel, p, Prow, zt_h, y.x, y.y, kk, g0, g1, K);
+  kept_drift(sel, p, Prow, zt_h, y.x, y.y, reinterpret_cast<uint16_t*>(kk),
+             reinterpret_cast<float*>(sk), g0, g1, K);
   const float G = warp_sum(g0 * g0 + g1 * g1);
   const float Kc = fmaxf(K, kEps);
   const float J = G / (Kc * Kc);
@@ -1000,8 +1172,9 @@ __global__ void __launch_bounds__(32 * kRowWarps, 9) k_score_rows(SelPtrs p, Bud
 // increases of J and track-best keeps the largest J.
 // MAXIMIZE: a maximising variant (keys are the increases of J, track-best keeps the largest
 // J), a template parameter so that the per-block key has no select.
-template <int MAXIMIZE>
-__global__ void __launch_bounds__(32 * kRowWarps, 10) k_round_rows(SelPtrs p, Budgets bud,
+// LARGE: some head swaps more than 32 blocks (warp_topm_large is compiled in, as in k_score_rows).
+template <int MAXIMIZE, bool LARGE>
+__global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 10) k_round_rows(SelPtrs p, Budgets bud,
                                                                   int round, float rho) {
   constexpr bool maximize = MAXIMIZE != 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1042,19 +1215,21 @@ __global__ void __launch_bounds__(32 * kRowWarps, 10) k_round_rows(SelPtrs p, Bu
       const float dG = inD ? fmaf(-2.0f * pv[u], tv[u], s2) : fmaf(2.0f * pv[u], tv[u], s2);
       const float dJ = delta_J(G, K, dG, inD ? pv[u] : -pv[u]);
       k4[u] = order_key(maximize ? -dJ : dJ);
-      if (j + u < p.ncand) top.add(k4[u], inD);
     }
+  }, [&](int j, const uint32_t (&k4)[4]) {
+    const uint32_t dword = Dw[j >> 5] >> (j & 31);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) top.add(k4[u], (dword >> u) & 1u);
   });
   // the swapped blocks as a list: written by the selection itself on the common path
   // (after the radix counters in the key area), else gathered from the bitmasks R and X
   uint16_t* lst = reinterpret_cast<uint16_t*>(kk + 256);
   int nl = 2 * m;
   bool listed = false;
-  if (m <= 64) {
-    listed = warp_topm_pair(kk, p.ncand, m, Dw, top, Rw, Xw, p.words, sk, si, lst);
+  if (!LARGE || m <= 64) {
+    listed = warp_topm_pair<LARGE>(kk, p.ncand, m, Dw, top, Rw, Xw, p.words, sk, si, lst);
   } else {
-    warp_topm(kk, p.ncand, m, Rw, p.words, sk, si, Dw, true);
-    warp_topm(kk, p.ncand, m, Xw, p.words, sk, si, Dw, false);
+    warp_topm_large<true>(kk, p.ncand, m, Dw, Rw, Xw, p.words, sk, si);
   }
   if (round == 0) {
     // both selections took m blocks from their side only if the drop set holds that many on
@@ -1092,7 +1267,10 @@ __global__ void __launch_bounds__(32 * kRowWarps, 10) k_round_rows(SelPtrs p, Bu
   const float2 y = *reinterpret_cast<const float2*>(p.ytil + ri * 64 + 2 * lane);
   const float2 gold = *reinterpret_cast<const float2*>(p.gtil + ri * 64 + 2 * lane);
   float g0 = gold.x, g1 = gold.y, Kn = K;
-  swap_drift_list(lst, nl, Prow, zt_h, y.x, y.y, g0, g1, Kn);
+  // the restored blocks join the kept set and the dropped ones leave it: g~ += sum_R P_k
+  // (z~_k - y~) - sum_X P_k (z~_k - y~) and K += sum_R P_k - sum_X P_k over the 2m swapped
+  // blocks (exactly the kept-set sums of Eq. 10-11 in exact arithmetic)
+  drift_sum(lst, nl, Prow, zt_h, y.x, y.y, reinterpret_cast<float*>(sk), g0, g1, Kn);
   const float Gn = warp_sum(g0 * g0 + g1 * g1);
   const float Kc = fmaxf(Kn, kEps);
   const float Jn = Gn / (Kc * Kc);
@@ -1510,7 +1688,12 @@ cudaError_t launch_score(const SelectArgs& a, cudaStream_t st) {
   if ((e = launch_drift_norms(a, st)) != cudaSuccess) return e;
   const size_t rsmem =
       (size_t)kRowWarps * warp_scratch_words(s.ld, score_mask_words(s.words, a.v.cdf > 0.f)) * 4;
-  auto kern = a.v.key == 0 ? k_score_rows<0> : a.v.key == 1 ? k_score_rows<1> : k_score_rows<2>;
+  int cmax = 0;
+  for (int h = 0; h < s.H; ++h) cmax = max(cmax, a.c[h]);
+  const bool large = cmax > 32 * kTopK;
+  auto kern = a.v.key == 0   ? (large ? k_score_rows<0, true> : k_score_rows<0, false>)
+              : a.v.key == 1 ? (large ? k_score_rows<1, true> : k_score_rows<1, false>)
+                             : (large ? k_score_rows<2, true> : k_score_rows<2, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
   if (e != cudaSuccess) return e;
   kern<<<dim3((s.nqc + kRowWarps - 1) / kRowWarps, s.H), 32 * kRowWarps, rsmem, st>>>(
@@ -1526,7 +1709,11 @@ cudaError_t launch_round(const SelectArgs& a, int round, float rho, cudaStream_t
   cudaError_t e = launch_gain(a, round, rho, st);  // t_ij on the tensor cores
   if (e != cudaSuccess) return e;
   const size_t rsmem = (size_t)kRowWarps * warp_scratch_words(s.ld, 3 * s.words) * 4;
-  auto kern = a.v.direction != 0 ? k_round_rows<1> : k_round_rows<0>;
+  int mmax = 0;
+  for (int h = 0; h < s.H; ++h) mmax = max(mmax, swap_count(a.c[h], s.ncand, round, rho));
+  const bool large = mmax > 32;
+  auto kern = a.v.direction != 0 ? (large ? k_round_rows<1, true> : k_round_rows<1, false>)
+                                 : (large ? k_round_rows<0, true> : k_round_rows<0, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
   if (e != cudaSuccess) return e;
   kern<<<dim3((s.nqc + kRowWarps - 1) / kRowWarps, s.H), 32 * kRowWarps, rsmem, st>>>(
