@@ -165,10 +165,13 @@ __global__ void __launch_bounds__(256) k_pairs(const int32_t* __restrict__ row_p
                                                int64_t cap, int64_t scratch_cap, int nb,
                                                int npairs, int H, bool qb128,
                                                int32_t* __restrict__ plist,
-                                               int32_t* __restrict__ plen, uint32_t* status) {
+                                               int32_t* __restrict__ plen, uint32_t* status,
+                                               uint32_t* counter) {
   __shared__ uint32_t bits[8][2][RESS_MAX_BLOCKS / 32];
+  pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pair = blockIdx.x * 8 + warp;
+  if (pair == 0 && lane == 0) *counter = 0u;  // the attention's tile counter
   if (pair >= H * npairs) return;
   const int h = pair / npairs, p = pair % npairs;
   const int words = (nb + 31) / 32;
@@ -199,6 +202,7 @@ __global__ void __launch_bounds__(256) k_pairs(const int32_t* __restrict__ row_p
     atomicOr((x < ea ? bA : bB) + (j >> 5), 1u << (j & 31));
   }
   __syncwarp();
+  pdl_trigger();
   // Entry order: the k-th block kept by the first query block only and the k-th kept by the
   // second only (k < P, the smaller of the two counts, both ascending) alternate at list
   // positions 2k, 2k + 1, so that the two halves' softmax work of consecutive one-sided
@@ -280,6 +284,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = S.tmem_base;
+  pdl_wait();
 
   if (warp == 0) {
     // =============================== producer ====================================
@@ -352,6 +357,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       ++it;
       q_loaded = false;
     }
+    pdl_trigger();  // no items left: the CTA ends with those in flight
     if (!failed) {
       const int s = g % kStages, u = g / kStages;
       if (u > 0 && !warp_wait(&S.kv_empty[s], (u - 1) & 1, abort)) {
@@ -726,14 +732,13 @@ cudaError_t launch_attn_pairs(const AttnArgs& x, cudaStream_t st) {
   const Shape& s = x.s;
   const int npairs = attn_num_pairs(s);
   const int pairs = s.H * npairs;
-  k_pairs<<<(pairs + 7) / 8, 256, 0, st>>>(x.row_ptr, x.col_idx, x.col_capacity, x.scratch_cap,
-                                           s.nb, npairs, s.H, s.qb == 128, x.plist, x.plen,
-                                           x.status);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_pairs, (pairs + 7) / 8, 256, 0, st, true, x.row_ptr, x.col_idx, x.col_capacity,
+                    x.scratch_cap, s.nb, npairs, s.H, s.qb == 128, x.plist, x.plen, x.status,
+                    x.counter);
 }
 
-cudaError_t launch_attn_range(const AttnArgs& x, int p0, int p1, int slot, cudaStream_t st) {
+cudaError_t launch_attn_range(const AttnArgs& x, int p0, int p1, int slot, bool overlap,
+                              cudaStream_t st) {
   const Shape& s = x.s;
   const int npairs = attn_num_pairs(s);
   if (p0 < 0 || p1 > npairs || p0 >= p1 || slot < 0 || slot >= kAttnCounterSlots)
@@ -769,16 +774,13 @@ cudaError_t launch_attn_range(const AttnArgs& x, int p0, int p1, int slot, cudaS
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int grid = min(items, 2 * sm_count());
-  kern<<<grid, kAttnThreads, smem, st>>>(tq, tk, tv, p);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, kAttnThreads, smem, st, overlap, tq, tk, tv, p);
 }
 
 cudaError_t launch_sparse_attn(const AttnArgs& x, cudaStream_t st) {
   cudaError_t e = launch_attn_pairs(x, st);
   if (e != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(x.counter, 0, sizeof(uint32_t), st)) != cudaSuccess) return e;
-  return launch_attn_range(x, 0, attn_num_pairs(x.s), 0, st);
+  return launch_attn_range(x, 0, attn_num_pairs(x.s), 0, true, st);
 }
 
 }  // namespace ress

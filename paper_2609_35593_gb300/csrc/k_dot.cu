@@ -89,7 +89,10 @@ __global__ void __launch_bounds__(kDotThreads)
     k_dot(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const __grid_constant__ CUtensorMap tmOut, const DotParams p) {
   const int h = blockIdx.z, i0 = blockIdx.y * kDotTile, j0 = blockIdx.x * kDotTile;
-  if (MODE == kDotGain && swap_count(p.bud.c[h], p.ncand, p.round, p.rho) <= 0) return;
+  if (MODE == kDotGain && swap_count(p.bud.c[h], p.ncand, p.round, p.rho) <= 0) {
+    pdl_wait();
+    return;
+  }
   extern __shared__ uint8_t smem_raw[];
   DotSmem& S = *reinterpret_cast<DotSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                            ~static_cast<uintptr_t>(1023));
@@ -105,14 +108,16 @@ __global__ void __launch_bounds__(kDotThreads)
     prefetch_tensormap(&tmB);
     prefetch_tensormap(&tmOut);
   }
-  if (MODE == kDotDist) {
-    const int j = j0 + (int)threadIdx.x;  // kDotThreads == kDotTile
-    S.bcol[threadIdx.x] = j < p.nb ? p.b[(int64_t)h * p.nb + j] : 0.f;
-  }
   if (warp == 0) tmem_alloc(&S.tmem_base, kDotCols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_wait();
+  if (MODE == kDotDist) {
+    const int j = j0 + (int)threadIdx.x;  // kDotThreads == kDotTile
+    S.bcol[threadIdx.x] = j < p.nb ? p.b[(int64_t)h * p.nb + j] : 0.f;
+    __syncthreads();
+  }
   const uint32_t tmem = S.tmem_base;
 
   bool issued = false;  // warp 0: MMAs went out (their completion must be awaited)
@@ -160,6 +165,7 @@ __global__ void __launch_bounds__(kDotThreads)
     }
   }
 
+  pdl_trigger();
   // ---- epilogue: warp w holds rows 32w .. 32w + 31 of the tile (TMEM lanes) ----------
   bool ok = dot_wait(&S.done, 0, abort, kDotWaitNs);
   if (!ok && lane == 0 && !*abort) {
@@ -322,9 +328,7 @@ cudaError_t launch_dot(const SelectArgs& a, int64_t a_terms, int64_t b_terms, in
       cudaFuncSetAttribute(k_dot<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((ncols + kDotTile - 1) / kDotTile, (s.nqc + kDotTile - 1) / kDotTile, s.H);
-  k_dot<MODE><<<grid, kDotThreads, smem, st>>>(ta, tb, to, p);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_dot<MODE>, grid, kDotThreads, smem, st, true, ta, tb, to, p);
 }
 
 }  // namespace

@@ -120,8 +120,7 @@ __global__ void __launch_bounds__(kOThreads, 1)
     k_oproj(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
             const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmX,
             const __grid_constant__ CUtensorMap tmY, const OParams p) {
-  const int ntile = tiles_of_cta<MODE>(p);
-  if (ntile == 0) return;
+  const int ntile = tiles_of_cta<MODE>(p);  // at least 1: the grid has at most one CTA per tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -159,6 +158,7 @@ __global__ void __launch_bounds__(kOThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = C.tmem_base;
+  pdl_wait();
 
   if (warp == 0) {
     // ================================ loads ==========================================
@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(kOThreads, 1)
         __syncwarp();
       }
     }
+    pdl_trigger();  // every slice of the CTA's tiles is on its way
     if (failed && lane == 0) {
       o_give_up(C, p.status);
       volatile int no_abort = 0;  // copies already issued land before the memory goes away
@@ -401,9 +402,7 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_oproj<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int grid = MODE == kDrift ? p.mtiles : min(p.mtiles * p.ntiles, sm_count_of_device());
-  k_oproj<MODE><<<grid, kOThreads, smem, st>>>(ta, ta2, tb, tx, ty, p);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_oproj<MODE>, grid, kOThreads, smem, st, true, ta, ta2, tb, tx, ty, p);
 }
 
 }  // namespace

@@ -112,9 +112,13 @@ __global__ void __launch_bounds__(kThreads) k_pool(const uint16_t* __restrict__ 
                                                     float* __restrict__ kbar,
                                                     float* __restrict__ vbar,
                                                     uint16_t* __restrict__ qsplit,
-                                                    uint16_t* __restrict__ ksplit) {
+                                                    uint16_t* __restrict__ ksplit,
+                                                    uint32_t* __restrict__ zero, int nzero) {
   __shared__ float part[kThreads * 8];
   const int j = blockIdx.x, which = blockIdx.y;
+  ptx::pdl_wait();
+  if (j == 0 && which == 0)  // k_yagg's arrival counters
+    for (int x = threadIdx.x; x < nzero; x += kThreads) zero[x] = 0u;
   const int bs = which == 0 ? qb : kBlock;        // tokens per block
   const int nblocks = which == 0 ? nq : nb;
   if (j >= nblocks) return;
@@ -144,6 +148,7 @@ __global__ void __launch_bounds__(kThreads) k_pool(const uint16_t* __restrict__ 
     for (int e = 0; e < 8; ++e) part[slot * C * 8 + c * 8 + e] = acc[e];
   }
   __syncthreads();
+  ptx::pdl_trigger();
   const float inv = 1.0f / (float)valid;
   for (int f = threadIdx.x; f < C * 8; f += kThreads) {
     float s = 0.f;
@@ -178,6 +183,7 @@ __global__ void __launch_bounds__(kThreads) k_zproj(const float* __restrict__ F,
   __shared__ float npart[8][4];
   const int h = blockIdx.y, j0 = blockIdx.x * 16, t = threadIdx.x;
   const int warp = t >> 5, lane = t & 31;
+  ptx::pdl_wait();
   for (int f = t; f < 1024; f += kThreads) {  // float4 units
     const int r = f >> 4, c4 = (f & 15) * 4;
     *reinterpret_cast<float4*>(&Fs[r][c4]) =
@@ -190,6 +196,7 @@ __global__ void __launch_bounds__(kThreads) k_zproj(const float* __restrict__ F,
     *reinterpret_cast<float4*>(&Vs[r][c4]) = v;
   }
   __syncthreads();
+  ptx::pdl_trigger();
   const int a = t & 63, q = t >> 6;  // q is uniform across a warp
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
@@ -1099,6 +1106,7 @@ template <int KEY, bool LARGE>
 __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(SelPtrs p, Budgets bud,
                                                                   Variant v) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  ptx::pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.y, i = blockIdx.x * kRowWarps + warp;
   if (i >= p.nqc) return;
@@ -1132,6 +1140,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(Se
     }
   }, [](int, const uint32_t (&)[4]) {});
   warp_topm<LARGE>(kk, p.ncand, bud.c[h], sel, p.words, sk, si, hist);  // sel = kept
+  ptx::pdl_trigger();
   // drop set D0 = candidates not kept
   for (int w = lane; w < p.words; w += 32) sel[w] = valid_bits(w, p.ncand) & ~sel[w];
   __syncwarp();
@@ -1178,6 +1187,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 10) k_round_rows(S
                                                                   int round, float rho) {
   constexpr bool maximize = MAXIMIZE != 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  ptx::pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int h = blockIdx.y, i = blockIdx.x * kRowWarps + warp;
   const int m = swap_count(bud.c[h], p.ncand, round, rho);
@@ -1256,6 +1266,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 10) k_round_rows(S
     }
     __syncwarp();
   }
+  ptx::pdl_trigger();
   // every listed block changes sides: restores leave D, drops join it
   for (int e = lane; e < nl; e += 32) {
     const int j = lst[e] & 0x7fff;
@@ -1305,6 +1316,7 @@ __global__ void __launch_bounds__(512) k_pairing(const uint32_t* __restrict__ bm
                                                  int words, int ncand, int npaired, int items,
                                                  int32_t* __restrict__ prow) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  ptx::pdl_wait();
   constexpr int W = kPairWindow;
   // kept sets as rows of 64-bit words with an odd row stride, so that the eight rows one
   // load touches fall in distinct bank pairs
@@ -1390,6 +1402,7 @@ __global__ void __launch_bounds__(512) k_pairing(const uint32_t* __restrict__ bm
     freeb &= ~matched_s[round & 1];
     if (t == 0) matched_s[(round + 1) & 1] = 0ull;  // read by every thread a round ago
   }
+  ptx::pdl_trigger();
   // pair slots in the order of the pairs' first blocks
   if (t < W) {
     const bool low = partner_s[t] > t;
@@ -1430,6 +1443,7 @@ struct CsrOut {
   const int32_t* prow;   // optional: rows of items u < npaired (k_pairing), else adjacent
   int npaired;
   uint32_t* status;
+  uint32_t* counters;    // optional: the attention's tile counters, cleared here
   int rows_per_item;     // 2 on the 64-token grid, 1 on the 128-token grid
   bool variable;         // row offsets from row_ptr (k_rowptr) instead of the fixed budgets
 };
@@ -1441,6 +1455,7 @@ __global__ void __launch_bounds__(1024) k_rowptr(const int32_t* __restrict__ kco
                                                  int nq, int nqc, int nb,
                                                  int32_t* __restrict__ row_ptr) {
   __shared__ long long wsum[32];
+  ptx::pdl_wait();
   const long long R = (long long)H * nq;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const long long per = (R + 1023) / 1024;
@@ -1482,7 +1497,10 @@ __device__ __forceinline__ void csr_write_word(const CsrOut& o, uint32_t bits, i
 }
 
 __global__ void k_csr(SelPtrs p, Budgets bud, CsrBases cb, int H, CsrOut o) {
+  ptx::pdl_wait();
   const int h = blockIdx.y, lane = threadIdx.x & 31;
+  if (o.counters && h == 0 && blockIdx.x == 0 && threadIdx.x < kAttnCounterSlots)
+    o.counters[threadIdx.x] = 0u;  // the attention's tile counters
   const int rpi = o.rows_per_item;
   const int items = (p.nq + rpi - 1) / rpi;
   const int u = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -1531,6 +1549,7 @@ __global__ void k_csr(SelPtrs p, Budgets bud, CsrBases cb, int H, CsrOut o) {
     }
     P = min(__reduce_add_sync(kFull, nA), __reduce_add_sync(kFull, nB));
   }
+  ptx::pdl_trigger();
   // Lane l owns word w0 + l of each row: warp scans of the lanes' counts give every word's
   // first list positions, then each lane writes the blocks of its own word.
   int posU = 0, cA = 0, cB = 0, cR = 0;
@@ -1671,16 +1690,14 @@ cudaError_t launch_score(const SelectArgs& a, cudaStream_t st) {
   float* kbar = (float*)(a.ws + a.L.kbar);
   float* vbar = (float*)(a.ws + a.L.vbar);
   float* ztil = (float*)(a.ws + a.L.ztil);
-  k_pool<<<dim3(s.nb, 3), kThreads, 0, st>>>(a.Q, a.K, a.V, s.N, s.H, s.nb, s.qb, s.nq, qbar,
-                                              kbar, vbar,
-                                              (uint16_t*)(a.ws + a.L.asplit),
-                                              (uint16_t*)(a.ws + a.L.ksplit));
-  note_launch();
-  k_zproj<<<dim3((s.nb + 15) / 16, s.H), kThreads, 0, st>>>(
-      a.F, vbar, s.nb, ztil, (uint16_t*)(a.ws + a.L.zsplit), (int64_t)s.H * s.nb * kHeadDim,
-      (float*)(a.ws + a.L.nz));
-  note_launch();
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_pool, dim3(s.nb, 3), kThreads, 0, st, true, a.Q, a.K, a.V, s.N, s.H,
+                             s.nb, s.qb, s.nq, qbar, kbar, vbar, (uint16_t*)(a.ws + a.L.asplit),
+                             (uint16_t*)(a.ws + a.L.ksplit), (uint32_t*)(a.ws + a.L.plen),
+                             yagg_arrivals(s));
+  if (e != cudaSuccess) return e;
+  e = launch_pdl(k_zproj, dim3((s.nb + 15) / 16, s.H), kThreads, 0, st, true, a.F, vbar, s.nb, ztil,
+                 (uint16_t*)(a.ws + a.L.zsplit), (int64_t)s.H * s.nb * kHeadDim,
+                 (float*)(a.ws + a.L.nz));
   if (e != cudaSuccess || s.ncand <= 0 || s.nqc <= 0) return e;
   // pooled logits, then P and y~, then q (Sec. 4.1, Eq. 1, Eq. 9), on the tensor cores
   if ((e = launch_logits(a, st)) != cudaSuccess) return e;
@@ -1696,10 +1713,8 @@ cudaError_t launch_score(const SelectArgs& a, cudaStream_t st) {
                              : (large ? k_score_rows<2, true> : k_score_rows<2, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((s.nqc + kRowWarps - 1) / kRowWarps, s.H), 32 * kRowWarps, rsmem, st>>>(
-      p, budgets_of(a), a.v);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3((s.nqc + kRowWarps - 1) / kRowWarps, s.H), 32 * kRowWarps, rsmem, st,
+                    true, p, budgets_of(a), a.v);
 }
 
 cudaError_t launch_round(const SelectArgs& a, int round, float rho, cudaStream_t st) {
@@ -1716,16 +1731,14 @@ cudaError_t launch_round(const SelectArgs& a, int round, float rho, cudaStream_t
                                  : (large ? k_round_rows<0, true> : k_round_rows<0, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
   if (e != cudaSuccess) return e;
-  kern<<<dim3((s.nqc + kRowWarps - 1) / kRowWarps, s.H), 32 * kRowWarps, rsmem, st>>>(
-      p, budgets_of(a), round, rho);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3((s.nqc + kRowWarps - 1) / kRowWarps, s.H), 32 * kRowWarps, rsmem, st,
+                    true, p, budgets_of(a), round, rho);
 }
 
 cudaError_t launch_csr(const SelectArgs& a, const int64_t* head_base, int32_t* row_ptr,
                        int32_t* col_idx, int64_t col_capacity, float* J_best,
                        uint32_t* drop_mask, int32_t* plist, int32_t* plen, int64_t plist_cap,
-                       const int32_t* prow, cudaStream_t st) {
+                       const int32_t* prow, uint32_t* counters, cudaStream_t st) {
   const Shape& s = a.s;
   SelPtrs p = sel_ptrs(s, a.ws, a.L);
   CsrBases cb;
@@ -1744,14 +1757,14 @@ cudaError_t launch_csr(const SelectArgs& a, const int64_t* head_base, int32_t* r
   o.variable = a.v.cdf > 0.f;
   o.prow = prow;
   o.npaired = prow ? paired_items(s) : 0;
+  o.counters = counters;
   if (o.variable) {
-    k_rowptr<<<1, 1024, 0, st>>>(p.kcount, s.H, s.nq, s.nqc, s.nb, row_ptr);
-    note_launch();
+    const cudaError_t e =
+        launch_pdl(k_rowptr, 1, 1024, 0, st, true, p.kcount, s.H, s.nq, s.nqc, s.nb, row_ptr);
+    if (e != cudaSuccess) return e;
   }
   const int items = (s.nq + o.rows_per_item - 1) / o.rows_per_item;
-  k_csr<<<dim3((items + 7) / 8, s.H), 256, 0, st>>>(p, budgets_of(a), cb, s.H, o);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_csr, dim3((items + 7) / 8, s.H), 256, 0, st, true, p, budgets_of(a), cb, s.H, o);
 }
 
 bool pairing_active(const Shape& s, const Variant& v) {
@@ -1767,10 +1780,9 @@ cudaError_t launch_pairing(const SelectArgs& a, int32_t* prow, cudaStream_t st) 
   const size_t smem = (size_t)kPairWindow * ((((s.words + 1) >> 1) | 1) * 8);
   cudaError_t e = cudaFuncSetAttribute(k_pairing, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_pairing<<<dim3(windows, s.H), 512, smem, st>>>((const uint32_t*)(a.ws + a.L.bmask), s.nq, s.words,
-                                                   s.ncand, npaired, (s.nb + 1) / 2, prow);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_pairing, dim3(windows, s.H), 512, smem, st, true,
+                    (const uint32_t*)(a.ws + a.L.bmask), s.nq, s.words, s.ncand, npaired,
+                    (s.nb + 1) / 2, prow);
 }
 
 }  // namespace ress

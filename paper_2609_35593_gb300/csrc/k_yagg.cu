@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kYThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_wait();
   const uint32_t tmem = S.tmem_base;
 
   if (warp == kMmaWarp) {
@@ -278,6 +279,7 @@ __global__ void __launch_bounds__(kYThreads, 1)
       if (lane == 0) mbar_arrive(&S.conv[s]);
     }
     if (failed && lane == 0) y_give_up(S, p.status);
+    pdl_trigger();
     // ---- epilogue: y~ row r, channels 16 qq .. 16 qq + 15 ------------------------------
     float nyp = 0.f;
     bool have = false;
@@ -370,7 +372,27 @@ __global__ void __launch_bounds__(kYThreads, 1)
   }
 }
 
+// One CTA per SM: when the stripes of rows leave SMs idle, split the key blocks into as many
+// parts (up to 3) as still run in one wave.  (A second wave costs more than the split saves:
+// measured at 32 views on 64-token query blocks, 96 stripes.)  The partial sums of k parts
+// take 64 k of the ld floats per row of the gains array.
+int yagg_parts(const Shape& s) {
+  const int stripes = (s.nqc + kYRows - 1) / kYRows, nchunks = (s.nb + kYChunk - 1) / kYChunk;
+  int dev = 0, sms = 1, parts = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  for (int k = 2; k <= 3 && k <= nchunks && 64 * k <= s.ld; ++k)
+    if ((int64_t)stripes * s.H * k <= sms) parts = k;
+  return parts;
+}
+
 }  // namespace
+
+// The counts live in the attention items' length array (H ceil(nb / 2) words, unused until
+// the lists are written); k_pool clears them.
+int yagg_arrivals(const Shape& s) {
+  return yagg_parts(s) > 1 ? (s.nqc + kYRows - 1) / kYRows * s.H : 0;
+}
 
 cudaError_t launch_yagg(const SelectArgs& a, cudaStream_t st) {
   const Shape& s = a.s;
@@ -393,31 +415,16 @@ cudaError_t launch_yagg(const SelectArgs& a, cudaStream_t st) {
   p.ny = (float*)(a.ws + a.L.ny);
   p.term_words = (int64_t)s.H * s.nq * 32;
   p.status = (uint32_t*)(a.ws + a.L.status);
-  // One CTA per SM: when the stripes of rows leave SMs idle, split the key blocks into as
-  // many parts (up to 3) as still run in one wave.  (A second wave costs more than the
-  // split saves: measured at 32 views on 64-token query blocks, 96 stripes.)
   const int stripes = (s.nqc + kYRows - 1) / kYRows;
-  int dev = 0, sms = 1;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  p.parts = 1;
-  // (the partial sums of k parts take 64 k of the ld floats per row of the gains array)
-  for (int k = 2; k <= 3 && k <= p.nchunks && 64 * k <= s.ld; ++k)
-    if ((int64_t)stripes * s.H * k <= sms) p.parts = k;
+  p.parts = yagg_parts(s);
   // scratch while the selection scores: the gains array (partial y~) and the attention
   // items' length array (arrival counts), both unused until the restoration rounds
   p.part_buf = (float*)(a.ws + a.L.t);
   p.arrivals = (uint32_t*)(a.ws + a.L.plen);
-  cudaError_t e;
-  if (p.parts > 1 &&
-      (e = cudaMemsetAsync(p.arrivals, 0, (size_t)stripes * s.H * sizeof(uint32_t), st)) != cudaSuccess)
-    return e;
   const size_t smem = sizeof(YSmem) + 1024;
-  e = cudaFuncSetAttribute(k_yagg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_yagg, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_yagg<<<dim3(stripes, s.H, p.parts), kYThreads, smem, st>>>(tl, tz, p);
-  note_launch();
-  return cudaGetLastError();
+  return launch_pdl(k_yagg, dim3(stripes, s.H, p.parts), kYThreads, smem, st, true, tl, tz, p);
 }
 
 }  // namespace ress

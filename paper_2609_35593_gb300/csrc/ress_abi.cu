@@ -308,7 +308,8 @@ static int restore_impl(const ress_dims* d, const int32_t* c_h, int32_t rounds, 
     if (ce != cudaSuccess) return cuda_fail(ce, "ress_restore pairing");
   }
   cudaError_t ce = ress::launch_csr(a, base, row_ptr, col_idx, col_capacity, J_best, drop_mask,
-                                    plist, plen, (int64_t)s.H * s.nq * s.ld, prow, st);
+                                    plist, plen, (int64_t)s.H * s.nq * s.ld, prow,
+                                    items ? reinterpret_cast<uint32_t*>(w + L.counter) : nullptr, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "ress_restore csr");
   return ok();
 }
@@ -424,8 +425,7 @@ int ress_forward(const ress_dims* d, const uint16_t* Q, const uint16_t* K, const
   ress::AttnArgs a = attn_args(s, L, Q, K, V, row_ptr, col_idx, col_capacity, O, false, ws);
   use_forward_pairing(&a, s, L, ws);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t ce = cudaMemsetAsync(a.counter, 0, sizeof(uint32_t), st);
-  if (ce == cudaSuccess) ce = ress::launch_attn_range(a, 0, ress::attn_num_pairs(s), 0, st);
+  cudaError_t ce = ress::launch_attn_range(a, 0, ress::attn_num_pairs(s), 0, true, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "ress_forward attention");
   return ok();
 }
@@ -480,8 +480,7 @@ int ress_forward_host(const ress_dims* d, const uint16_t* Q_host, const uint16_t
   OverlapStreams* o = nullptr;
   cudaError_t ce = overlap_streams(&o);
   if (ce != cudaSuccess) return cuda_fail(ce, "ress_forward_host streams");
-  if ((ce = cudaMemsetAsync(a.counter, 0, kOutChunks * sizeof(uint32_t), st)) != cudaSuccess ||
-      (ce = cudaEventRecord(o->ready, st)) != cudaSuccess ||
+  if ((ce = cudaEventRecord(o->ready, st)) != cudaSuccess ||
       (ce = cudaStreamWaitEvent(o->aux, o->ready, 0)) != cudaSuccess)
     return cuda_fail(ce, "ress_forward_host attention");
   const int np = ress::attn_num_pairs(s);
@@ -500,7 +499,7 @@ int ress_forward_host(const ress_dims* d, const uint16_t* Q_host, const uint16_t
     cudaStream_t cs = (c & 1) ? o->aux : st;
     const int64_t t0 = 128 * (int64_t)p0;
     const int64_t t1 = 128 * (int64_t)p1 < d->n_tokens ? 128 * (int64_t)p1 : d->n_tokens;
-    if ((ce = ress::launch_attn_range(a, p0, p1, c, cs)) == cudaSuccess &&
+    if ((ce = ress::launch_attn_range(a, p0, p1, c, false, cs)) == cudaSuccess &&
         (ce = cudaEventRecord(o->done[c], cs)) == cudaSuccess &&
         (ce = cudaStreamWaitEvent(o->copy, o->done[c], 0)) == cudaSuccess)
       ce = cudaMemcpyAsync(reinterpret_cast<char*>(O_host) + t0 * row_bytes,

@@ -151,6 +151,29 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
 // Counts one kernel launch of this library (host side, process-wide; ress_kernel_launches).
 void note_launch();
 
+// Launches a kernel that may start before the kernel ahead of it in the stream has finished
+// (programmatic dependent launch), so that its launch and its set-up (barriers, TMEM,
+// constants in shared memory) overlap the other's last CTAs; see ptx::pdl_wait for what the
+// kernel has to do.  One forward is 15 launches: 2 views 122 -> 91 us, 8 views 337 -> 306 us,
+// 32 views 1384 -> 1357 us.  overlap = false: an ordinary launch of the same kernel.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       bool overlap, const A&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  note_launch();
+  return e;
+}
+
 // Kernel launchers (defined in k_select.cu / k_attn.cu); each returns a cudaError_t.
 // Selection variant (ress_variant) as the kernels take it.
 struct Variant {
@@ -177,13 +200,15 @@ cudaError_t launch_gain(const SelectArgs& a, int round, float rho, cudaStream_t 
 cudaError_t launch_logits(const SelectArgs& a, cudaStream_t st);
 cudaError_t launch_drift_norms(const SelectArgs& a, cudaStream_t st);
 cudaError_t launch_yagg(const SelectArgs& a, cudaStream_t st);
+// Arrival counters of launch_yagg that must be zero when it runs (0: none; see k_yagg).
+int yagg_arrivals(const Shape& s);
 // Kept-block lists in CSR form; with plist set, also the attention items' union lists and
-// their lengths (what launch_attn_pairs builds from a caller's CSR), so that a forward can
-// go straight to launch_attn_range.
+// their lengths (what launch_attn_pairs builds from a caller's CSR), and clears the attention's
+// tile counters, so that a forward can go straight to launch_attn_range.
 cudaError_t launch_csr(const SelectArgs& a, const int64_t* head_base, int32_t* row_ptr,
                        int32_t* col_idx, int64_t col_capacity, float* J_best,
                        uint32_t* drop_mask, int32_t* plist, int32_t* plen, int64_t plist_cap,
-                       const int32_t* prow, cudaStream_t st);
+                       const int32_t* prow, uint32_t* counters, cudaStream_t st);
 // Attention items of a forward on the 64-token grid with fixed budgets: the candidate query
 // blocks are paired by the overlap of their best kept lists, within windows of
 // kPairWindow blocks (prow, see ress_ws_layout); items of the window hold pair indices
@@ -212,13 +237,14 @@ struct AttnArgs {
 cudaError_t launch_sparse_attn(const AttnArgs& a, cudaStream_t st);
 // The two halves of launch_sparse_attn, for callers that split the attention: the union
 // lists of the query-block pairs, then the attention over pairs [p0, p1) of every head
-// (query tokens [128 p0, 128 p1)) with tile-scheduler counter `slot`, which the caller
-// zeroes before the launch.  Pairs are 128 query rows: two 64-token query blocks, or one
+// (query tokens [128 p0, 128 p1)) with tile-scheduler counter `slot`, which the union pass (or
+// the CSR kernel of a forward) has cleared.  overlap: see launch_pdl.  Pairs are 128 query rows: two 64-token query blocks, or one
 // 128-token block on the paper's grid.
 constexpr int kAttnCounterSlots = 16;  // uint32 counters in the workspace's 64-byte slot
 int attn_num_pairs(const Shape& s);
 cudaError_t launch_attn_pairs(const AttnArgs& a, cudaStream_t st);
-cudaError_t launch_attn_range(const AttnArgs& a, int p0, int p1, int slot, cudaStream_t st);
+cudaError_t launch_attn_range(const AttnArgs& a, int p0, int p1, int slot, bool overlap,
+                              cudaStream_t st);
 
 struct OProjArgs {
   int N, H, Dm;                      // tokens, heads (K = 64 H), d_model
