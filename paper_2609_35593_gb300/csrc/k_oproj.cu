@@ -4,22 +4,33 @@
 // O is [N, K] with K = H * 64 (the concatenated head outputs), W_o is [d_model, K] (Linear
 // weight, out x in), x and y are [N, d_model].
 //
-// One tile = 128 tokens x 256 output channels, reduced over K in 64-wide slices through a
-// three-stage TMA ring (128-byte swizzle, both operands K-major).  192 threads:
-//   warp 0     TMA of the O and W_o slices (the drift variant loads O_a and O_b slices);
-//   warp 1     TMEM owner; one elected lane of the converged warp issues per slice 4 x
-//              tcgen05.mma M128 N256 K16 (the drift variant: 4 into each of two accumulators);
-//   warps 2-5  epilogue, row r = TMEM lane: residual update: the tile's x (loaded by TMA into
+// One tile = 256 tokens x 256 output channels of a CTA pair (cta_group::2: M256 N256 K16, each
+// CTA holding 128 of A's rows, 128 of B's rows and 128 rows of the accumulator), reduced over K
+// in 64-wide slices through a TMA ring (128-byte swizzle, both operands K-major).  What bounds
+// the kernel is operand delivery into the SM (about 50 bytes per cycle): a pair brings 32 KB per
+// SM and slice for the 128 x 256 x 64 products of one CTA, where a CTA by itself needs 48 KB
+// (43,968 tokens, K = d_model = 1024: 86.9 us with single CTAs, 78.5 with pairs, 74.2 with the
+// epilogue on eight warps instead of four; 1.24 PFLOP/s, and the tensor pipe's clock under its
+// power limit is the next bound: with half of every load left out it still took 62 us).  Per CTA 320 threads:
+//   warp 0     TMA of its half of the O and W_o slices (the drift variant loads O_a and O_b
+//              slices); the bytes of both CTAs are counted by the barrier of the rank-0 CTA;
+//   warp 1     TMEM owner; in the rank-0 CTA one elected lane of the converged warp issues per
+//              slice 4 MMAs for the pair (the drift variant: 4 into each of two accumulators);
+//   warps 2-9  epilogue, row r = TMEM lane, four warps per half of the channels: residual update: the tile's x (loaded by TMA into
 //              a swizzled staging area) plus the accumulator, rounded to bf16 in place and
 //              written out by TMA bulk stores; drift: the squared difference of the two
 //              accumulators summed over the row's channels, then over each block's 64 rows
 //              in a fixed order.
-// The residual update runs persistent CTAs over the tiles with two TMEM accumulators, so a
-// tile's epilogue overlaps the next tile's MMAs; the drift variant gives each CTA one
-// 128-token stripe and walks its channel tiles in order.
+// The residual update runs persistent pairs over the tiles with two TMEM accumulators, so a
+// tile's epilogue overlaps the next tile's MMAs; the drift variant gives each 256-token stripe
+// to a cluster of one, two or four pairs, which take its channel tiles in turn and add up
+// their rows' sums through distributed shared memory.
 // Every mbarrier wait is bounded; a wait that gives up records RESS_ETIMEOUT, makes the CTA
-// leave its loops together, lets copies and MMAs already issued finish (again bounded), frees
-// TMEM and returns.
+// leave its loops (and, as its waits run out, the other one), lets copies and MMAs already
+// issued finish (again bounded); the pair then meets at a cluster barrier, frees TMEM and
+// returns.
+
+#include <climits>
 
 #include <cudaTypedefs.h>
 
@@ -33,38 +44,42 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 
 namespace {
 
-constexpr int kOThreads = 192;
-constexpr int kOM = 128;                      // tokens per tile
+constexpr int kOThreads = 320;
+constexpr int kOM = 128;                      // tokens per tile and CTA
 constexpr int kON = 256;                      // output channels per tile
-constexpr int kOStages = 3;
 constexpr uint32_t kABytes = kOM * 128;       // 128 x 64 bf16
-constexpr uint32_t kBBytes = kON * 128;       // 256 x 64 bf16
+constexpr uint32_t kBBytes = kON / 2 * 128;   // 128 x 64 bf16: this CTA's half of B's rows
 constexpr uint32_t kOCols = 512;              // TMEM: two 128 x 256 fp32 accumulators
 constexpr uint64_t kOWaitNs = 2000000000ull;  // 2 s per wait
 constexpr uint64_t kODrainNs = 200000000ull;  // 0.2 s to drain after an abort
 
 enum { kResidual = 0, kDrift = 1 };
 
-// Shared-memory layout.  Residual: A[3] | B[3] | X (4 boxes of 128 x 64 bf16).
-// Drift: A[3] | A2[3] | B[3].
-constexpr uint32_t kOffA = 0;
-constexpr uint32_t kOffB = kOStages * kABytes;                 // residual
-constexpr uint32_t kOffX = kOffB + kOStages * kBBytes;
-constexpr uint32_t kOffA2 = kOStages * kABytes;                // drift
-constexpr uint32_t kOffB2 = kOffA2 + kOStages * kABytes;
-constexpr uint32_t kOData = kOffX + 4 * 16384;                 // the larger of the two layouts
-static_assert(kOffB2 + kOStages * kBBytes <= kOData, "drift layout fits the residual one");
+// Shared-memory layout.  Residual: five stages of A | B, then X (4 boxes of 128 x 64 bf16).
+// Drift: four stages of A | A2 | B.
+template <int MODE>
+constexpr int kOStages = MODE == kDrift ? 4 : 5;
+template <int MODE>
+constexpr uint32_t kStageBytes = (MODE == kDrift ? 2 : 1) * kABytes + kBBytes;
+constexpr uint32_t kOffX = kOStages<kResidual> * kStageBytes<kResidual>;
+constexpr uint32_t kOData = kOffX + 4 * 16384;  // the larger of the two layouts
+static_assert(kOStages<kDrift> * kStageBytes<kDrift> <= kOData, "drift layout fits the residual one");
 
 struct OCtl {
-  float rowsum[kOM];
-  uint64_t full[kOStages], empty[kOStages], acc_full[2], acc_empty[2], x_full;
+  float rowsum[2][kOM];
+  float blocksum[4];
+  uint64_t full[5], empty[5], acc_full[2], acc_empty[2], x_full[2];
   uint32_t tmem_base;
   int abort;
 };
 
 struct OParams {
   int N, K, Dm, nb;
-  int mtiles, ntiles;
+  int mtiles, ntiles;  // tiles of 256 tokens, of 256 channels
+  // residual: the first `whole` tiles run whole; each one after them as `parts` units of
+  // 256 / parts channels
+  int whole, parts;
+  int group;  // drift: pairs per stripe (cluster of 2 group CTAs), at most ntiles
   bool has_x;
   float* drift;
   uint32_t* status;
@@ -84,43 +99,51 @@ __device__ __forceinline__ void o_give_up(OCtl& C, uint32_t* status) {
   *reinterpret_cast<volatile int*>(&C.abort) = 1;
 }
 
-// Named barrier of the four epilogue warps that also ANDs a flag across them.
-__device__ __forceinline__ bool o_epi_sync_and(bool v) {
+// Named barriers of the four epilogue warps of channel half hf (0 or 1); the first also ANDs
+// a flag across them.
+__device__ __forceinline__ bool o_epi_sync_and(int hf, bool v) {
   uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      "bar.red.and.pred q, %2, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"(v ? 1u : 0u)
+      : "r"(v ? 1u : 0u), "r"(1 + hf)
       : "memory");
   return r != 0;
 }
-__device__ __forceinline__ void o_epi_sync() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+__device__ __forceinline__ void o_epi_sync(int hf) {
+  asm volatile("bar.sync %0, 128;" ::"r"(3 + hf) : "memory");
+}
 
+// One unit of work: rows of stripe mt, channels [col, col + width).
+struct OUnit {
+  int mt, col, width;
+};
+// Drift: a cluster of p.group pairs per stripe, which take its channel tiles in turn.
 template <int MODE>
-__device__ __forceinline__ int tiles_of_cta(const OParams& p) {
-  if (MODE == kDrift) return p.ntiles;
-  const int total = p.mtiles * p.ntiles;
-  return blockIdx.x < total ? (total - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+__device__ __forceinline__ int units_of_pair(const OParams& p) {
+  if (MODE == kDrift) return (p.ntiles - 1 - (int)(cluster_rank() >> 1)) / p.group + 1;
+  const int units = p.whole + (p.mtiles * p.ntiles - p.whole) * p.parts;
+  return (units - 1 - (int)(blockIdx.x >> 1)) / (int)(gridDim.x >> 1) + 1;
 }
 template <int MODE>
-__device__ __forceinline__ void tile_coords(const OParams& p, int k, int& mt, int& nt) {
-  if (MODE == kDrift) {
-    mt = blockIdx.x;
-    nt = k;
-  } else {  // consecutive tiles share their token stripe, so O slices are re-read from L2
-    const int t = blockIdx.x + k * gridDim.x;
-    mt = t / p.ntiles;
-    nt = t % p.ntiles;
-  }
+__device__ __forceinline__ OUnit unit_of_pair(const OParams& p, int k) {
+  if (MODE == kDrift)
+    return OUnit{(int)blockIdx.x / (2 * p.group), kON * ((int)(cluster_rank() >> 1) + k * p.group), kON};
+  // consecutive tiles share their token stripe, so O slices are re-read from L2
+  const int u = (int)(blockIdx.x >> 1) + k * (int)(gridDim.x >> 1);
+  if (u < p.whole) return OUnit{u / p.ntiles, kON * (u % p.ntiles), kON};
+  const int t = p.whole + (u - p.whole) / p.parts, w = kON / p.parts;
+  return OUnit{t / p.ntiles, kON * (t % p.ntiles) + w * ((u - p.whole) % p.parts), w};
 }
 
 template <int MODE>
 __global__ void __launch_bounds__(kOThreads, 1)
     k_oproj(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-            const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmX,
+            const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmBpart,
+            const __grid_constant__ CUtensorMap tmX,
             const __grid_constant__ CUtensorMap tmY, const OParams p) {
-  const int ntile = tiles_of_cta<MODE>(p);  // at least 1: the grid has at most one CTA per tile
+  const int nunits = units_of_pair<MODE>(p);  // at least 1: at most one pair per unit
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -128,21 +151,25 @@ __global__ void __launch_bounds__(kOThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort = &C.abort;
   const int ksteps = p.K / 64;
-  auto A = [&](int s) { return base + kOffA + s * kABytes; };
-  auto A2 = [&](int s) { return base + kOffA2 + s * kABytes; };
-  auto B = [&](int s) { return base + (MODE == kDrift ? kOffB2 : kOffB) + s * kBBytes; };
+  constexpr int kStages = kOStages<MODE>;
+  const int rank = (int)cluster_rank() & 1;   // this CTA's half of the pair's rows
+  const int lead = (int)cluster_rank() & ~1;  // the pair's rank-0 CTA
+  const uint32_t both = 3u << lead;
+  auto A = [&](int s) { return base + s * kStageBytes<MODE>; };
+  auto A2 = [&](int s) { return A(s) + kABytes; };
+  auto B = [&](int s) { return A(s) + (MODE == kDrift ? 2 : 1) * kABytes; };
   uint8_t* X = base + kOffX;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kOStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&C.full[s], 1);
       mbar_init(&C.empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&C.acc_full[b], 1);
-      mbar_init(&C.acc_empty[b], 4);
+      mbar_init(&C.acc_empty[b], 16);  // the epilogue warps of both CTAs
+      mbar_init(&C.x_full[b], 1);
     }
-    mbar_init(&C.x_full, 1);
     C.abort = 0;
     fence_barrier_init();
     prefetch_tensormap(&tmA);
@@ -153,48 +180,62 @@ __global__ void __launch_bounds__(kOThreads, 1)
       if (p.has_x) prefetch_tensormap(&tmX);
     }
   }
-  if (warp == 1) tmem_alloc(&C.tmem_base, kOCols);
+  if (warp == 1) tmem_alloc_pair(&C.tmem_base, kOCols);
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // both CTAs' barriers exist
   tc_fence_after();
   const uint32_t tmem = C.tmem_base;
   pdl_wait();
 
   if (warp == 0) {
     // ================================ loads ==========================================
-    const uint32_t bytes = (MODE == kDrift ? 2 * kABytes : kABytes) + kBBytes;
+    // the barriers of the rank-0 CTA count the bytes of both
     int it = 0;
     bool failed = false;
-    for (int k = 0; k < ntile && !failed; ++k) {
-      int mt, nt;
-      tile_coords<MODE>(p, k, mt, nt);
+    for (int k = 0; k < nunits && !failed; ++k) {
+      const OUnit t = unit_of_pair<MODE>(p, k);
+      // the stripe of the pair's next unit into L2 while this one runs (by the pair that takes
+      // the stripe's first channels): 69.4 -> 67.4 us at 43,968 tokens
+      const OUnit t2 = unit_of_pair<MODE>(p, min(k + 1, nunits - 1));
+      const bool ahead = MODE == kResidual && k + 1 < nunits && t2.col == 0;
       for (int ks = 0; ks < ksteps; ++ks, ++it) {
-        const int s = it % kOStages, u = it / kOStages;
+        const int s = it % kStages, u = it / kStages;
         if (u > 0 && !o_wait(&C.empty[s], (u - 1) & 1, abort)) {
           failed = true;
           break;
         }
         if (lane == 0) {
-          mbar_arrive_expect_tx(&C.full[s], bytes);
-          tma_load_3d(A(s), &tmA, &C.full[s], 64 * ks, kOM * mt, 0);
-          if (MODE == kDrift) tma_load_3d(A2(s), &tmA2, &C.full[s], 64 * ks, kOM * mt, 0);
-          tma_load_3d(B(s), &tmB, &C.full[s], 64 * ks, kON * nt, 0);
+          const uint32_t bytes = (MODE == kDrift ? 2 : 1) * kABytes + t.width / 2 * 128;
+          if (rank == 0) mbar_arrive_expect_tx(&C.full[s], 2 * bytes);
+          const uint32_t full = cluster_addr(&C.full[s], lead);
+          const int row = kOM * (2 * t.mt + rank);
+          tma_load_3d_pair(A(s), &tmA, full, 64 * ks, row, 0);
+          if (MODE == kDrift) tma_load_3d_pair(A2(s), &tmA2, full, 64 * ks, row, 0);
+          tma_load_3d_pair(B(s), t.width == kON ? &tmB : &tmBpart, full, 64 * ks,
+                           t.col + t.width / 2 * rank, 0);
+          if (ahead) tma_prefetch_3d(&tmA, 64 * ks, kOM * (2 * t2.mt + rank), 0);
         }
         __syncwarp();
       }
     }
     pdl_trigger();  // every slice of the CTA's tiles is on its way
+    // the pair's MMAs release every stage in both CTAs: nothing arrives here after the end
+    for (int q = max(0, it - kStages); q < it && !failed; ++q)
+      if (!o_wait(&C.empty[q % kStages], (q / kStages) & 1, abort)) failed = true;
     if (failed && lane == 0) {
       o_give_up(C, p.status);
-      volatile int no_abort = 0;  // copies already issued land before the memory goes away
-      for (int q = max(0, it - kOStages); q < it; ++q)
-        mbar_wait(&C.full[q % kOStages], (q / kOStages) & 1, &no_abort, kODrainNs);
+      volatile int no_abort = 0;  // copies already issued land before the memory goes away (the
+      // rank-1 CTA's are counted in the other one: its waits here just run out)
+      for (int q = max(0, it - kStages); q < it; ++q)
+        mbar_wait(&C.full[q % kStages], (q / kStages) & 1, &no_abort, kODrainNs);
     }
     __syncwarp();
+  } else if (warp == 1 && rank == 1) {
+    // the rank-0 CTA issues the pair's MMAs
   } else if (warp == 1) {
     // ================================ MMAs ===========================================
     const bool leader = elect_one();
-    const uint32_t idesc = idesc_bf16_f32(kOM, kON, false);
     int it = 0;
     bool failed = false;
     if (__popc(__ballot_sync(0xffffffffu, leader)) != 1) {  // exactly one issuing lane
@@ -204,7 +245,8 @@ __global__ void __launch_bounds__(kOThreads, 1)
       }
       failed = true;
     }
-    for (int k = 0; k < ntile && !failed; ++k) {
+    for (int k = 0; k < nunits && !failed; ++k) {
+      const uint32_t idesc = idesc_bf16_f32(2 * kOM, unit_of_pair<MODE>(p, k).width, false);
       const int b = MODE == kDrift ? 0 : (k & 1);
       const int use = MODE == kDrift ? k : (k >> 1);  // earlier uses of accumulator b
       if (use > 0 && !o_wait(&C.acc_empty[b], (use - 1) & 1, abort)) {
@@ -214,8 +256,8 @@ __global__ void __launch_bounds__(kOThreads, 1)
       tc_fence_after();
       const uint32_t acc = tmem + (MODE == kDrift ? 0u : (uint32_t)kON * b);
       for (int ks = 0; ks < ksteps; ++ks, ++it) {
-        const int s = it % kOStages;
-        if (!o_wait(&C.full[s], (it / kOStages) & 1, abort)) {
+        const int s = it % kStages;
+        if (!o_wait(&C.full[s], (it / kStages) & 1, abort)) {
           failed = true;
           break;
         }
@@ -224,17 +266,17 @@ __global__ void __launch_bounds__(kOThreads, 1)
           const uint32_t a = smem_u32(A(s)), bb = smem_u32(B(s));
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            mma_bf16_ss(acc, sdesc_sw128(a + 32 * kk), sdesc_sw128(bb + 32 * kk), idesc,
+            mma_bf16_ss_pair(acc, sdesc_sw128(a + 32 * kk), sdesc_sw128(bb + 32 * kk), idesc,
                         (ks > 0 || kk > 0) ? 1u : 0u);
           if (MODE == kDrift) {
             const uint32_t a2 = smem_u32(A2(s));
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              mma_bf16_ss(tmem + kON, sdesc_sw128(a2 + 32 * kk), sdesc_sw128(bb + 32 * kk), idesc,
+              mma_bf16_ss_pair(tmem + kON, sdesc_sw128(a2 + 32 * kk), sdesc_sw128(bb + 32 * kk), idesc,
                           (ks > 0 || kk > 0) ? 1u : 0u);
           }
-          mma_commit(&C.empty[s]);
-          if (ks + 1 == ksteps) mma_commit(&C.acc_full[b]);
+          mma_commit_pair(&C.empty[s], both);
+          if (ks + 1 == ksteps) mma_commit_pair(&C.acc_full[b], both);
         }
         __syncwarp();
       }
@@ -244,39 +286,54 @@ __global__ void __launch_bounds__(kOThreads, 1)
       if (it > 0) {  // MMAs still running must finish before TMEM is freed
         volatile int no_abort = 0;
         const int q = it - 1;
-        mbar_wait(&C.empty[q % kOStages], (q / kOStages) & 1, &no_abort, kODrainNs);
+        mbar_wait(&C.empty[q % kStages], (q / kStages) & 1, &no_abort, kODrainNs);
       }
     }
     __syncwarp();
   } else {
     // ================================ epilogue =======================================
+    // two groups of four warps, each a half of the tile's channels with its own staging
+    // boxes, x barrier and stores
+    const int hf = (warp - 2) >> 2;
     const int quarter = warp & 3;
     const int r = 32 * quarter + lane;  // row of the tile = TMEM lane
-    const uint32_t lane_base = (uint32_t)(32 * quarter) << 16;
-    const bool leader = (warp == 2 && lane == 0);
+    const uint32_t lane_base = ((uint32_t)(32 * quarter) << 16) + kON / 2 * hf;
+    const bool leader = (warp - 2) % 4 == 0 && lane == 0;
+    uint8_t* Xh = X + 2 * hf * 16384;
     float rowsum = 0.f;
-    if (MODE == kResidual && p.has_x && leader) {  // the first tile's x
-      int mt, nt;
-      tile_coords<MODE>(p, 0, mt, nt);
-      mbar_arrive_expect_tx(&C.x_full, 4 * 16384);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) tma_load_3d(X + q * 16384, &tmX, &C.x_full, kON * nt + 64 * q, kOM * mt, 0);
-    }
-    for (int k = 0; k < ntile; ++k) {
-      int mt, nt;
-      tile_coords<MODE>(p, k, mt, nt);
+    // 64-channel boxes of this half in a unit (a part of a tile may have none)
+    auto boxes_of = [&](const OUnit& t) { return max(0, min(2, t.width / 64 - 2 * hf)); };
+    auto load_x = [&](int k) {  // this half of unit k's x into the staging boxes
+      const OUnit t = unit_of_pair<MODE>(p, k);
+      const int boxes = boxes_of(t);
+      if (boxes == 0) return;
+      mbar_arrive_expect_tx(&C.x_full[hf], boxes * 16384);
+      for (int q = 0; q < boxes; ++q)
+        tma_load_3d(Xh + q * 16384, &tmX, &C.x_full[hf], t.col + kON / 2 * hf + 64 * q,
+                    kOM * (2 * t.mt + rank), 0);
+    };
+    if (MODE == kResidual && p.has_x && leader) load_x(0);
+    for (int k = 0; k < nunits; ++k) {
+      const OUnit t = unit_of_pair<MODE>(p, k);
+      const int boxes = boxes_of(t);
+      const int row0 = kOM * (2 * t.mt + rank), col0 = t.col + kON / 2 * hf;
       const int b = MODE == kDrift ? 0 : (k & 1);
       const int use = MODE == kDrift ? k : (k >> 1);
+      if (MODE == kResidual && p.has_x && leader && k + 1 < nunits) {  // the next unit's x into L2
+        const OUnit t2 = unit_of_pair<MODE>(p, k + 1);
+        for (int q = 0; q < boxes_of(t2); ++q)
+          tma_prefetch_3d(&tmX, t2.col + kON / 2 * hf + 64 * q, kOM * (2 * t2.mt + rank), 0);
+      }
       bool ok = o_wait(&C.acc_full[b], use & 1, abort);
-      if (MODE == kResidual && p.has_x && ok) ok = o_wait(&C.x_full, k & 1, abort);
-      if (!o_epi_sync_and(ok)) {  // the four warps leave together
+      if (MODE == kResidual && p.has_x && ok && boxes > 0) ok = o_wait(&C.x_full[hf], k & 1, abort);
+      if (!o_epi_sync_and(hf, ok)) {  // the four warps leave together
         if (!ok && lane == 0) o_give_up(C, p.status);
         break;
       }
       tc_fence_after();
       if (MODE == kDrift) {
 #pragma unroll 1
-        for (int q = 0; q < kON / 32; ++q) {
+        for (int q = 0; q < kON / 64; ++q) {
           uint32_t va[32], vb[32];
           RESS_TMEM_LD32(tmem + lane_base + 32 * q, va);
           RESS_TMEM_LD32(tmem + kON + lane_base + 32 * q, vb);
@@ -289,10 +346,10 @@ __global__ void __launch_bounds__(kOThreads, 1)
       } else {
         const uint32_t acc = tmem + (uint32_t)kON * b + lane_base;
 #pragma unroll 1
-        for (int q = 0; q < kON / 32; ++q) {  // channels 32q .. 32q + 31: box q/2, chunks 4(q%2)..
+        for (int q = 0; q < 2 * boxes; ++q) {  // channels 32q .. 32q + 31: box q/2, chunks 4(q%2)..
           uint32_t v[32];
           RESS_TMEM_LD32(acc + 32 * q, v);
-          uint8_t* row = X + (q >> 1) * 16384 + r * 128;
+          uint8_t* row = Xh + (q >> 1) * 16384 + r * 128;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint4* at = reinterpret_cast<uint4*>(row + (((4 * (q & 1) + c) ^ (r & 7)) << 4));
@@ -310,46 +367,49 @@ __global__ void __launch_bounds__(kOThreads, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&C.acc_empty[b]);  // the accumulator may be reused
+      if (lane == 0) mbar_arrive_cluster(cluster_addr(&C.acc_empty[b], lead));  // may be reused
       if (MODE == kResidual) {
         fence_proxy_async_smem();
-        o_epi_sync();
+        o_epi_sync(hf);
         if (leader) {
 #pragma unroll 1
-          for (int q = 0; q < 4; ++q)
-            if (kON * nt + 64 * q < p.Dm) tma_store_3d(&tmY, X + q * 16384, kON * nt + 64 * q, kOM * mt, 0);
+          for (int q = 0; q < boxes; ++q)
+            if (col0 + 64 * q < p.Dm && row0 < p.N)
+              tma_store_3d(&tmY, Xh + q * 16384, col0 + 64 * q, row0, 0);
           bulk_commit();
-          bulk_wait_read_all();  // the staging area is free again
-          if (p.has_x && k + 1 < ntile) {
-            int mt2, nt2;
-            tile_coords<MODE>(p, k + 1, mt2, nt2);
-            mbar_arrive_expect_tx(&C.x_full, 4 * 16384);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              tma_load_3d(X + q * 16384, &tmX, &C.x_full, kON * nt2 + 64 * q, kOM * mt2, 0);
-          }
+          bulk_wait_read_all();  // the staging boxes are free again
+          if (p.has_x && k + 1 < nunits) load_x(k + 1);
         }
       }
     }
-    if (MODE == kDrift) {
-      C.rowsum[r] = rowsum;
-      o_epi_sync();
-      if (threadIdx.x - 64 < 2) {  // one thread per 64-token block of the stripe, rows in order
-        const int blk = 2 * blockIdx.x + (threadIdx.x - 64);
-        if (blk < p.nb && !*abort) {
-          float s = 0.f;
-          for (int q = 0; q < 64; ++q) s += C.rowsum[64 * (threadIdx.x - 64) + q];
-          p.drift[blk] = s;
-        }
-      }
-    }
+    if (MODE == kDrift) C.rowsum[hf][r] = rowsum;
     if (leader) bulk_wait_read_all();
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // the pair's MMAs and barrier arrivals are over in both CTAs
+  if (MODE == kDrift) {
+    // the cluster's first pair sums its rows over the pairs (and their channel halves) in
+    // order, then each 64-token block over its rows, warp tree by warp tree
+    if (cluster_rank() < 2 && threadIdx.x < kOM) {
+      float v = 0.f;
+      for (int g = 0; g < p.group; ++g)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf)
+          v += ld_cluster_f32(cluster_addr(&C.rowsum[hf][threadIdx.x], 2 * g + rank));
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) C.blocksum[warp] = v;
+    }
+    cluster_sync();  // the other CTAs' sums have been read
+    if (cluster_rank() < 2 && threadIdx.x < 2) {
+      const int blk = 2 * (2 * ((int)blockIdx.x / (2 * p.group)) + rank) + (int)threadIdx.x;
+      if (blk < p.nb && !*abort) p.drift[blk] = C.blocksum[2 * threadIdx.x] + C.blocksum[2 * threadIdx.x + 1];
+    }
+  }
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kOCols);
+    tmem_dealloc_pair(tmem, kOCols);
   }
 }
 
@@ -377,8 +437,8 @@ int sm_count_of_device() {
 template <int MODE>
 cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   const int K = a.H * 64;
-  CUtensorMap ta, ta2, tb, tx, ty;
-  if (!make_bf16_map(&ta, a.O, a.N, K, kOM) || !make_bf16_map(&tb, a.W_o, a.Dm, K, kON))
+  CUtensorMap ta, ta2, tb, tbp, tx, ty;
+  if (!make_bf16_map(&ta, a.O, a.N, K, kOM) || !make_bf16_map(&tb, a.W_o, a.Dm, K, kON / 2))
     return cudaErrorInvalidValue;
   ta2 = ta;
   tx = ta;
@@ -393,7 +453,7 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   p.K = K;
   p.Dm = a.Dm;
   p.nb = (a.N + 63) / 64;
-  p.mtiles = (a.N + kOM - 1) / kOM;
+  p.mtiles = (a.N + 2 * kOM - 1) / (2 * kOM);
   p.ntiles = (a.Dm + kON - 1) / kON;
   p.has_x = a.x != nullptr;
   p.drift = a.drift;
@@ -401,8 +461,40 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   const size_t smem = kOData + sizeof(OCtl) + 1024;
   cudaError_t e = cudaFuncSetAttribute(k_oproj<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int grid = MODE == kDrift ? p.mtiles : min(p.mtiles * p.ntiles, sm_count_of_device());
-  return launch_pdl(k_oproj<MODE>, grid, kOThreads, smem, st, true, ta, ta2, tb, tx, ty, p);
+  const int tiles = p.mtiles * p.ntiles, slots = max(1, sm_count_of_device() / 2);
+  // Tiles past the last whole wave of pairs run as 2 or 4 units of fewer channels each where
+  // those fit into one wave (43,968 tokens and d_model 1024: 688 tiles on 76 pairs are nine
+  // waves and four tiles: 68.3 us with a tenth wave, 67.7 split).
+  p.whole = tiles;
+  p.parts = 1;
+  const int left = tiles % slots;
+  if (MODE == kResidual && left > 0 && 2 * left <= slots) {
+    p.whole = tiles - left;
+    p.parts = 4 * left <= slots ? 4 : 2;
+  }
+  const int units = p.whole + (tiles - p.whole) * p.parts;
+  // Drift: as many pairs per stripe (a cluster) as make the fewest tiles in a row per SM; a
+  // GPC rarely has room for as many clusters of 8 CTAs as its SMs would allow, so those are
+  // counted with one in eight less (8 views: 43 stripes of 4 tiles leave 66 of 152 SMs idle
+  // with one pair each: 45.3 us, 41.2 with four; 16 views 89.8 and, with two, 73.1).
+  p.group = 1;
+  if (MODE == kDrift) {
+    int best = INT_MAX;
+    for (int g = 1; g <= 4 && g <= p.ntiles; g *= 2) {
+      const int fit = max(1, g == 4 ? slots * 7 / 32 : slots / g);
+      const int rounds = (p.mtiles + fit - 1) / fit * ((p.ntiles + g - 1) / g);
+      if (rounds < best) {
+        best = rounds;
+        p.group = g;
+      }
+    }
+  }
+  const int ctas = 2 * (MODE == kDrift ? p.mtiles * p.group : min(units, slots));
+  tbp = tb;
+  if (p.parts > 1 && !make_bf16_map(&tbp, a.W_o, a.Dm, K, kON / 2 / p.parts))
+    return cudaErrorInvalidValue;
+  return launch_pdl_cluster(k_oproj<MODE>, ctas, kOThreads, smem, st, 2 * p.group, ta, ta2, tb, tbp, tx,
+                            ty, p);
 }
 
 }  // namespace

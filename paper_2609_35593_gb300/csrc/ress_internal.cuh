@@ -157,21 +157,41 @@ void note_launch();
 // kernel has to do.  One forward is 15 launches: 2 views 122 -> 91 us, 8 views 337 -> 306 us,
 // 32 views 1384 -> 1357 us.  overlap = false: an ordinary launch of the same kernel.
 template <typename... P, typename... A>
-cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                       bool overlap, const A&... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_with(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                        bool overlap, int cluster, const A&... args) {
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster;
+    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1 : 0;
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
   note_launch();
   return e;
+}
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       bool overlap, const A&... args) {
+  return launch_with(kern, grid, block, smem, st, overlap, 1, args...);
+}
+// The same with clusters of `cluster` CTAs.
+template <typename... P, typename... A>
+cudaError_t launch_pdl_cluster(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                               cudaStream_t st, int cluster, const A&... args) {
+  return launch_with(kern, grid, block, smem, st, true, cluster, args...);
 }
 
 // Kernel launchers (defined in k_select.cu / k_attn.cu); each returns a cudaError_t.
