@@ -62,6 +62,8 @@ constexpr int kNO = 80;  // O columns: 64 output channels, the row sum, 15 unuse
 constexpr uint64_t kWaitNs = 2000000000ull;  // 2 s per wait
 constexpr uint64_t kDrainNs = 200000000ull;  // 0.2 s to drain after an abort
 constexpr int kFirst = 1, kLast = 2, kTerm = 4;
+constexpr int kMaxSplit = 4;   // CTAs per item in the split kernel
+constexpr int kPartStride = 68;  // floats per row there: 64 channels, row sum, maximum, 2 of padding
 constexpr int kItemSlots = 4;  // items announced to the softmax warps ahead of their tiles
 constexpr uint32_t kTileBytes = 64 * 128;    // one 64 x 64 bf16 tile
 // log2 units: rescale only when the running max grows by more than 2^20.  P is bf16 and O
@@ -99,6 +101,7 @@ struct AttnParams {
   const int32_t* plen;   // [H * npairs]
   const int32_t* prow;   // items p < npaired: query blocks a | b << 16 (64-token grid), or NULL
   int npaired;
+  int split;             // CTAs (a cluster) per item, 1: persistent CTAs over the items
   void* O;               // bf16 or float32 [N, H, 64]
   uint32_t* status;
   uint32_t* counter;
@@ -241,7 +244,13 @@ __global__ void __launch_bounds__(256) k_pairs(const int32_t* __restrict__ row_p
 // ------------------------------------------------------------------------------------
 // main kernel
 // ------------------------------------------------------------------------------------
-template <bool kOutF32>
+// kSplit: a cluster of a.split CTAs per item, CTA s of it taking its share of the item's list
+// (entries [n s / split, n (s + 1) / split)) as if that were the whole list.  Each row's O, row
+// sum and reference maximum then go to shared memory, and every CTA adds up a share of the
+// channels over the cluster: O = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s.  For layers
+// with fewer items than half the CTA slots, where the longest item (a dense one) alone would
+// set the kernel's time: see attn_split.
+template <bool kOutF32, bool kSplit>
 __global__ void __launch_bounds__(kAttnThreads, 2)
     k_attn(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
            const __grid_constant__ CUtensorMap tmV, const AttnParams a) {
@@ -285,6 +294,17 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   tc_fence_after();
   const uint32_t tmem = S.tmem_base;
   pdl_wait();
+  // this CTA's entries of an item's list
+  auto list_of = [&](int h, int p, int& n) -> const int32_t* {
+    const int32_t* lst = a.plist + a.row_ptr[(int64_t)h * a.rows_per_head + a.row_step * p];
+    n = a.plen[h * a.npairs + p];
+    if (kSplit) {
+      const int s = (int)cluster_rank(), lo = n * s / a.split;
+      n = n * (s + 1) / a.split - lo;
+      lst += lo;
+    }
+    return lst;
+  };
 
   if (warp == 0) {
     // =============================== producer ====================================
@@ -306,14 +326,21 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     };
     for (;;) {
       int item = 0;
-      if (lane == 0) item = (int)atomicAdd(a.counter, 1u);
-      item = __shfl_sync(0xffffffffu, item, 0);
+      if (kSplit) {  // the cluster's one item
+        if (it > 0 || pub > 0) break;
+        item = (int)blockIdx.x / a.split;
+      } else {
+        if (lane == 0) item = (int)atomicAdd(a.counter, 1u);
+        item = __shfl_sync(0xffffffffu, item, 0);
+      }
       if (item >= a.nitems) break;
-      int h, p;
+      int h, p, n;
       item_pair(a, item, h, p);
-      const int n = a.plen[h * a.npairs + p];
-      if (n <= 0) continue;
-      const int32_t* lst = a.plist + a.row_ptr[(int64_t)h * a.rows_per_head + a.row_step * p];
+      const int32_t* lst = list_of(h, p, n);
+      if (n <= 0) {
+        if (kSplit) break;
+        continue;
+      }
       if (!publish(item)) {
         failed = true;
         break;
@@ -522,6 +549,8 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     };
     int g = 0;
     bool stop = false;
+    float* part = reinterpret_cast<float*>(S.K[0]) + kPartStride * r;  // kSplit: this row's share
+    bool have = false;
     for (int pub = 0; !stop; ++pub) {
       const int slot = pub % kItemSlots;
       if (!warp_wait(&S.it_full[slot], (pub / kItemSlots) & 1, abort)) {
@@ -532,11 +561,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       __syncwarp();
       if (lane == 0) mbar_arrive(&S.it_empty[slot]);
       if (item < 0) break;
-      int h, p, t0, t1;
+      int h, p, t0, t1, n;
       item_pair(a, item, h, p);
       item_tokens(a, h, p, t0, t1);
-      const int n = a.plen[h * a.npairs + p];
-      const int32_t* lst = a.plist + a.row_ptr[(int64_t)h * a.rows_per_head + a.row_step * p];
+      const int32_t* lst = list_of(h, p, n);
       float m_use = -INFINITY;  // this row's reference maximum (log2 units); warp-uniform -inf
       int mine = lane < n ? lst[lane] : 0;
       for (int e0 = 0; e0 < n && !stop; e0 += 32) {
@@ -643,7 +671,16 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
             RESS_TMEM_LD32(tmem + lane_base + kColO + 32, o[1]);
             RESS_TMEM_LD16(tmem + lane_base + kColO + 64, ls);
             const float l = __uint_as_float(ls[0]);  // row sum of the bf16 probabilities
-            if (row_exists) {
+            if (kSplit) {  // K's stages are free: every copy has landed and every MMA is done
+              have = true;
+#pragma unroll
+              for (int c = 0; c < 64; c += 4)
+                *reinterpret_cast<float4*>(part + c) = make_float4(
+                    __uint_as_float(o[c >> 5][c & 31]), __uint_as_float(o[c >> 5][(c + 1) & 31]),
+                    __uint_as_float(o[c >> 5][(c + 2) & 31]), __uint_as_float(o[c >> 5][(c + 3) & 31]));
+              part[64] = l;
+              part[65] = m_use;
+            } else if (row_exists) {
               if (!(l > 0.f)) flag_status(a.status, kStatusBadRow);
               const float inv = l > 0.f ? 1.0f / l : 0.f;
               const int64_t off = ((int64_t)token * a.H + h) * 64;
@@ -679,11 +716,60 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
         mine = nxt;
       }
     }
+    if (kSplit && !have) {  // no entries for this CTA
+#pragma unroll
+      for (int c = 0; c < 64; ++c) part[c] = 0.f;
+      part[64] = 0.f;
+      part[65] = -INFINITY;
+    }
   }
 
   __syncwarp();
   tc_fence_before();
   __syncthreads();
+  if (kSplit) {
+    cluster_sync();  // every CTA's rows are in its shared memory
+    if (warp >= 2) {
+      const int r = (warp & 3) * 32 + lane;
+      int h, p, t0, t1;
+      item_pair(a, (int)blockIdx.x / a.split, h, p);
+      item_tokens(a, h, p, t0, t1);
+      const int token = (r >> 6 ? t1 : t0) + (r & 63);
+      if (token < a.N) {
+        const float* row = reinterpret_cast<const float*>(S.K[0]) + kPartStride * r;
+        float m = -INFINITY, l = 0.f;
+        for (int s = 0; s < a.split; ++s) m = fmaxf(m, ld_cluster_f32(cluster_addr(row + 65, s)));
+        float w[kMaxSplit];
+#pragma unroll
+        for (int s = 0; s < kMaxSplit; ++s) {
+          w[s] = 0.f;
+          if (s < a.split) {
+            const float ms = ld_cluster_f32(cluster_addr(row + 65, s));
+            w[s] = ms == -INFINITY ? 0.f : ex2(ms - m);
+            l = fmaf(w[s], ld_cluster_f32(cluster_addr(row + 64, s)), l);
+          }
+        }
+        if (!(l > 0.f)) flag_status(a.status, kStatusBadRow);
+        const float inv = l > 0.f ? 1.0f / l : 0.f;
+        const int s0 = (int)cluster_rank();
+        uint2* dst = reinterpret_cast<uint2*>(static_cast<uint16_t*>(a.O) + ((int64_t)token * a.H + h) * 64);
+        for (int c = 16 * s0 / a.split; c < 16 * (s0 + 1) / a.split; ++c) {  // four channels each
+          float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int s = 0; s < kMaxSplit; ++s)
+            if (s < a.split) {
+              const float4 v = ld_cluster_f32x4(cluster_addr(row + 4 * c, s));
+              o.x = fmaf(w[s], v.x, o.x);
+              o.y = fmaf(w[s], v.y, o.y);
+              o.z = fmaf(w[s], v.z, o.z);
+              o.w = fmaf(w[s], v.w, o.w);
+            }
+          dst[c] = make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
+        }
+      }
+    }
+    cluster_sync();  // the other CTAs have read this one's rows
+  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
@@ -728,6 +814,18 @@ static int sm_count() {
 
 int attn_num_pairs(const Shape& s) { return (s.nb + 1) / 2; }
 
+// CTAs per item of a forward's attention: with fewer items than half the CTA slots (two per
+// SM), as many as fit, up to 4.  Only the forward on the 64-token grid, whose output is not
+// tied bit for bit to ress_sparse_attn's (a share has its own reference maxima).  Lists below
+// 16 blocks gain nothing.  The whole layer with 1 / 2 / 3 / 4 CTAs per item: 2 views (88 items)
+// 89.8 / 85.7 / 85.3 / 100.8 us; 5,003 tokens x 3 heads (120 items, dense ones of 79 tiles) 106.7 /
+// 95.6 / 104.5 / 108.9; 8 views (1,376 items) 309.9 and, with two, 391.5: what does not fit into
+// one wave loses.
+int attn_split(const Shape& s) {
+  if (s.qb != kBlock || s.nb < 16) return 1;
+  return max(1, min(kMaxSplit, 2 * sm_count() / (s.H * attn_num_pairs(s))));
+}
+
 cudaError_t launch_attn_pairs(const AttnArgs& x, cudaStream_t st) {
   const Shape& s = x.s;
   const int npairs = attn_num_pairs(s);
@@ -770,9 +868,13 @@ cudaError_t launch_attn_range(const AttnArgs& x, int p0, int p1, int slot, bool 
   p.status = x.status;
   p.counter = x.counter + slot;
   const size_t smem = sizeof(AttnSmem) + 1024;
-  auto kern = x.out_f32 ? k_attn<true> : k_attn<false>;
+  p.split = x.split;
+  const bool split = x.split > 1;
+  auto kern = x.out_f32 ? k_attn<true, false> : split ? k_attn<false, true> : k_attn<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  if (split)
+    return launch_with(kern, items * x.split, kAttnThreads, smem, st, overlap, x.split, tq, tk, tv, p);
   const int grid = min(items, 2 * sm_count());
   return launch_pdl(kern, grid, kAttnThreads, smem, st, overlap, tq, tk, tv, p);
 }

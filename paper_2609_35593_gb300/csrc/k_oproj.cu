@@ -493,8 +493,8 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   tbp = tb;
   if (p.parts > 1 && !make_bf16_map(&tbp, a.W_o, a.Dm, K, kON / 2 / p.parts))
     return cudaErrorInvalidValue;
-  return launch_pdl_cluster(k_oproj<MODE>, ctas, kOThreads, smem, st, 2 * p.group, ta, ta2, tb, tbp, tx,
-                            ty, p);
+  return launch_with(k_oproj<MODE>, ctas, kOThreads, smem, st, true, 2 * p.group, ta, ta2, tb, tbp, tx,
+                     ty, p);
 }
 
 }  // namespace

@@ -351,14 +351,17 @@ static ress::AttnArgs attn_args(const ress::Shape& s, const ress_ws_layout& L,
   a.plist = reinterpret_cast<int32_t*>(w + L.t);  // the gains buffer is free during attention
   a.plen = reinterpret_cast<int32_t*>(w + L.plen);
   a.scratch_cap = (int64_t)s.H * s.nq * s.ld;  // entries of the t array
-  a.prow = nullptr;  // adjacent query blocks; a forward sets its pairing table
+  a.prow = nullptr;  // adjacent query blocks; a forward sets its pairing table and its split
   a.npaired = 0;
+  a.split = 1;
   return a;
 }
 
-// The attention of a forward uses the item table its CSR step wrote (ReSS, no variant).
+// The attention of a forward uses the item table its CSR step wrote (ReSS, no variant), and
+// several CTAs per item where the layer is small.
 static void use_forward_pairing(ress::AttnArgs* a, const ress::Shape& s, const ress_ws_layout& L,
                                 void* ws) {
+  a->split = ress::attn_split(s);
   if (ress::pairing_active(s, ress::Variant{0, 0, 0ull, 0.0f})) {
     a->prow = reinterpret_cast<const int32_t*>(static_cast<char*>(ws) + L.prow);
     a->npaired = ress::paired_items(s);
@@ -693,6 +696,7 @@ extern "C" int ress_sparse_attn_noalloc(const ress_dims* d, const uint16_t* Q, c
   a.scratch_cap = list_entries;
   a.prow = nullptr;  // items of adjacent query blocks
   a.npaired = 0;
+  a.split = 1;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t ce = ress::launch_sparse_attn(a, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "ress_sparse_attn_noalloc");

@@ -158,18 +158,18 @@ void note_launch();
 // 32 views 1384 -> 1357 us.  overlap = false: an ordinary launch of the same kernel.
 template <typename... P, typename... A>
 cudaError_t launch_with(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                        bool overlap, int cluster, const A&... args) {
+                        bool overlap, dim3 cluster, const A&... args) {
   cudaLaunchAttribute attr[2];
   int n = 0;
   if (overlap) {
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n++].val.programmaticStreamSerializationAllowed = 1;
   }
-  if (cluster > 1) {
+  if (cluster.x * cluster.y * cluster.z > 1) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
-    attr[n].val.clusterDim.x = (unsigned)cluster;
-    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
-    ++n;
+    attr[n].val.clusterDim.x = cluster.x;
+    attr[n].val.clusterDim.y = cluster.y;
+    attr[n++].val.clusterDim.z = cluster.z;
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
@@ -185,13 +185,7 @@ cudaError_t launch_with(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, 
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                        bool overlap, const A&... args) {
-  return launch_with(kern, grid, block, smem, st, overlap, 1, args...);
-}
-// The same with clusters of `cluster` CTAs.
-template <typename... P, typename... A>
-cudaError_t launch_pdl_cluster(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
-                               cudaStream_t st, int cluster, const A&... args) {
-  return launch_with(kern, grid, block, smem, st, true, cluster, args...);
+  return launch_with(kern, grid, block, smem, st, overlap, dim3(1), args...);
 }
 
 // Kernel launchers (defined in k_select.cu / k_attn.cu); each returns a cudaError_t.
@@ -253,6 +247,7 @@ struct AttnArgs {
   int64_t scratch_cap;
   const int32_t* prow;  // item table of a paired forward (items p < npaired), or NULL
   int npaired;
+  int split;            // CTAs per item (attn_split; bf16 output only)
 };
 cudaError_t launch_sparse_attn(const AttnArgs& a, cudaStream_t st);
 // The two halves of launch_sparse_attn, for callers that split the attention: the union
@@ -262,6 +257,7 @@ cudaError_t launch_sparse_attn(const AttnArgs& a, cudaStream_t st);
 // 128-token block on the paper's grid.
 constexpr int kAttnCounterSlots = 16;  // uint32 counters in the workspace's 64-byte slot
 int attn_num_pairs(const Shape& s);
+int attn_split(const Shape& s);  // CTAs per item of a forward's attention (k_attn.cu)
 cudaError_t launch_attn_pairs(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_attn_range(const AttnArgs& a, int p0, int p1, int slot, bool overlap,
                               cudaStream_t st);
