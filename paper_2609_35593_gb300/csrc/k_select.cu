@@ -353,10 +353,11 @@ __device__ void select_exact(const uint32_t* keys, const uint16_t* idx, int n, i
   const int lane = threadIdx.x & 31;
   auto part = [&](int x) { return idx != nullptr || takes_part(member, want, x); };
   uint32_t lo = 0;
+#pragma unroll 1
   for (int bit = 31; bit >= 0; --bit) {
     const uint32_t cand = lo | (1u << bit);
     int cnt = 0;
-#pragma unroll 4
+#pragma unroll 1
     for (int x = lane; x < n; x += 32) cnt += (keys[x] >= cand && part(x)) ? 1 : 0;
     cnt = __reduce_add_sync(kFull, cnt);
     if (cnt >= m) {
@@ -365,11 +366,12 @@ __device__ void select_exact(const uint32_t* keys, const uint16_t* idx, int n, i
     }
   }
   int gt = 0;
-#pragma unroll 4
+#pragma unroll 1
   for (int x = lane; x < n; x += 32) gt += (keys[x] > lo && part(x)) ? 1 : 0;
   gt = __reduce_add_sync(kFull, gt);
   const int need = m - gt;
   int taken = 0;
+#pragma unroll 1
   for (int x0 = 0; x0 < n; x0 += 32) {
     const int x = x0 + lane;
     const bool in = x < n && part(x);
@@ -761,10 +763,11 @@ __device__ __forceinline__ uint32_t mth_of_64(uint32_t a, uint32_t b, int m) {
 // positions); each side then selects exactly (radix select on its survivors).
 // Returns true when the chosen blocks went to lst (restores at lst[0..m), drops at
 // lst[m..2m) with bit 15 set) instead of the bitmasks; lst lies in the key area after its
-// first 256 words (the radix counters).  Above m = 32 the bound is loose (the m-th of only 64
-// values) and the survivors often overflow their 128 places per side; LARGE kernels then select
-// on all keys with warp_topm_large (m = 53 over 2142 keys at 100 views: 1611 us for the round
-// with the bit-by-bit search, 724 us with it).
+// first 256 words (the radix counters).  Above m = 20 or so the bound is loose (the m-th of only 64
+// values) and the survivors sometimes overflow their 128 places per side; LARGE kernels then
+// select on all keys with warp_topm_large (100 views, 2142 keys: m = 53 1611 us for the round
+// with the bit-by-bit search, 724 us with it; m = 26 463 and 427 us; at 64 views m = 21 takes
+// 174 us either way).
 template <bool LARGE>
 __device__ bool warp_topm_pair(const uint32_t* kk, int n, int m, const uint32_t* Dw,
                                const LaneTop2& top, uint32_t* selD, uint32_t* selB,
@@ -829,27 +832,30 @@ __device__ bool warp_topm_pair(const uint32_t* kk, int n, int m, const uint32_t*
     cntB += total >> 16;
   }
   __syncwarp();
-  if (cntD <= kHalf && cntB <= kHalf) {
-    // the keys are no longer needed: their first 256 words hold the radix counters
-    select_radix(sk, si, cntD, m, const_cast<uint32_t*>(kk), selD, lst, 0);
-    select_radix(sk + kHalf, si + kHalf, cntB, m, const_cast<uint32_t*>(kk), selB, lst + m, 0x8000);
-    __syncwarp();
-    return true;
-  }
-  if (LARGE) {
+  const bool listed = cntD <= kHalf && cntB <= kHalf;
+  if (LARGE && !listed) {
     warp_topm_large<true>(kk, n, m, Dw, selD, selB, words, sk, si);
     return false;
   }
-  if (cntD > kHalf)
-    select_exact(kk, nullptr, n, m, Dw, true, selD);
-  else
-    select_exact(sk, si, cntD, m, nullptr, true, selD);
-  if (cntB > kHalf)
-    select_exact(kk, nullptr, n, m, Dw, false, selB);
-  else
-    select_exact(sk + kHalf, si + kHalf, cntB, m, nullptr, true, selB);
+  // one copy of each selection for both sides: the kernel waits on instruction fetch (108 KB of
+  // code with a copy per side, 58 KB so; the 32-view layer's first round 62.9 -> 59.9 us)
+#pragma unroll 1
+  for (int t = 0; t < 2; ++t) {
+    const int cnt = t ? cntB : cntD;
+    const uint32_t* st = sk + kHalf * t;
+    const uint16_t* it = si + kHalf * t;
+    uint32_t* sel = t ? selB : selD;
+    if (listed) {
+      // the keys are no longer needed: their first 256 words hold the radix counters
+      select_radix(st, it, cnt, m, const_cast<uint32_t*>(kk), sel, lst + m * t, t ? 0x8000 : 0);
+    } else {
+      const bool over = cnt > kHalf;
+      select_exact(over ? kk : st, over ? nullptr : it, over ? n : cnt, m, over ? Dw : nullptr, t == 0,
+                   sel);
+    }
+  }
   __syncwarp();
-  return false;
+  return listed;
 }
 
 // g~ of row ri (this lane's channels 2 lane, 2 lane + 1), its three bf16 terms (the A
@@ -1181,7 +1187,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(Se
 // increases of J and track-best keeps the largest J.
 // MAXIMIZE: a maximising variant (keys are the increases of J, track-best keeps the largest
 // J), a template parameter so that the per-block key has no select.
-// LARGE: some head swaps more than 32 blocks (warp_topm_large is compiled in, as in k_score_rows).
+// LARGE: some head swaps more than 20 blocks (warp_topm_large is compiled in, as in k_score_rows).
 template <int MAXIMIZE, bool LARGE>
 __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 10) k_round_rows(SelPtrs p, Budgets bud,
                                                                   int round, float rho) {
@@ -1726,7 +1732,7 @@ cudaError_t launch_round(const SelectArgs& a, int round, float rho, cudaStream_t
   const size_t rsmem = (size_t)kRowWarps * warp_scratch_words(s.ld, 3 * s.words) * 4;
   int mmax = 0;
   for (int h = 0; h < s.H; ++h) mmax = max(mmax, swap_count(a.c[h], s.ncand, round, rho));
-  const bool large = mmax > 32;
+  const bool large = mmax > 20;
   auto kern = a.v.direction != 0 ? (large ? k_round_rows<1, true> : k_round_rows<1, false>)
                                  : (large ? k_round_rows<0, true> : k_round_rows<0, false>);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rsmem);
