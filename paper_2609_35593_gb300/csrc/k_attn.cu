@@ -101,7 +101,7 @@ struct AttnParams {
   const int32_t* plen;   // [H * npairs]
   const int32_t* prow;   // items p < npaired: query blocks a | b << 16 (64-token grid), or NULL
   int npaired;
-  int split;             // CTAs (a cluster) per item, 1: persistent CTAs over the items
+  int split, share;      // CTAs of a cluster, CTAs per sparse item (kSplit; else 1: persistent CTAs)
   void* O;               // bf16 or float32 [N, H, 64]
   uint32_t* status;
   uint32_t* counter;
@@ -244,10 +244,23 @@ __global__ void __launch_bounds__(256) k_pairs(const int32_t* __restrict__ row_p
 // ------------------------------------------------------------------------------------
 // main kernel
 // ------------------------------------------------------------------------------------
-// kSplit: a cluster of a.split CTAs per item, CTA s of it taking its share of the item's list
-// (entries [n s / split, n (s + 1) / split)) as if that were the whole list.  Each row's O, row
+// Which item a CTA of the split kernel works on, and which share of it: clusters of a.split CTAs
+// take one item with dense query blocks each, then the sparse items, a.share CTAs per item.
+struct Share {
+  int item, first, s, parts;  // CTA s of the item's `parts`, cluster ranks first .. first + parts - 1
+};
+__device__ __forceinline__ Share share_of_cta(const AttnParams& a) {
+  const int ndense = a.H * max(0, a.p1 - max(a.p0, a.nsparse));
+  const int c = (int)blockIdx.x / a.split, rank = (int)cluster_rank();
+  if (c < ndense) return Share{c, 0, rank, a.split};
+  const int k = rank / a.share;
+  return Share{ndense + (c - ndense) * (a.split / a.share) + k, k * a.share, rank % a.share, a.share};
+}
+
+// kSplit: several CTAs of a cluster per item, CTA s of `parts` taking its share of the item's
+// list (entries [n s / parts, n (s + 1) / parts)) as if that were the whole list.  Each row's O, row
 // sum and reference maximum then go to shared memory, and every CTA adds up a share of the
-// channels over the cluster: O = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s.  For layers
+// channels over the item's CTAs: O = sum_s 2^(m_s - m) O_s / sum_s 2^(m_s - m) l_s.  For layers
 // with fewer items than half the CTA slots, where the longest item (a dense one) alone would
 // set the kernel's time: see attn_split.
 template <bool kOutF32, bool kSplit>
@@ -299,8 +312,9 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
     const int32_t* lst = a.plist + a.row_ptr[(int64_t)h * a.rows_per_head + a.row_step * p];
     n = a.plen[h * a.npairs + p];
     if (kSplit) {
-      const int s = (int)cluster_rank(), lo = n * s / a.split;
-      n = n * (s + 1) / a.split - lo;
+      const Share c = share_of_cta(a);
+      const int lo = n * c.s / c.parts;
+      n = n * (c.s + 1) / c.parts - lo;
       lst += lo;
     }
     return lst;
@@ -328,7 +342,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
       int item = 0;
       if (kSplit) {  // the cluster's one item
         if (it > 0 || pub > 0) break;
-        item = (int)blockIdx.x / a.split;
+        item = share_of_cta(a).item;
       } else {
         if (lane == 0) item = (int)atomicAdd(a.counter, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
@@ -729,36 +743,37 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
   __syncthreads();
   if (kSplit) {
     cluster_sync();  // every CTA's rows are in its shared memory
-    if (warp >= 2) {
+    const Share my = share_of_cta(a);
+    if (warp >= 2 && my.item < a.nitems) {
       const int r = (warp & 3) * 32 + lane;
       int h, p, t0, t1;
-      item_pair(a, (int)blockIdx.x / a.split, h, p);
+      item_pair(a, my.item, h, p);
       item_tokens(a, h, p, t0, t1);
       const int token = (r >> 6 ? t1 : t0) + (r & 63);
       if (token < a.N) {
         const float* row = reinterpret_cast<const float*>(S.K[0]) + kPartStride * r;
         float m = -INFINITY, l = 0.f;
-        for (int s = 0; s < a.split; ++s) m = fmaxf(m, ld_cluster_f32(cluster_addr(row + 65, s)));
+        for (int s = 0; s < my.parts; ++s)
+          m = fmaxf(m, ld_cluster_f32(cluster_addr(row + 65, my.first + s)));
         float w[kMaxSplit];
 #pragma unroll
         for (int s = 0; s < kMaxSplit; ++s) {
           w[s] = 0.f;
-          if (s < a.split) {
-            const float ms = ld_cluster_f32(cluster_addr(row + 65, s));
+          if (s < my.parts) {
+            const float ms = ld_cluster_f32(cluster_addr(row + 65, my.first + s));
             w[s] = ms == -INFINITY ? 0.f : ex2(ms - m);
-            l = fmaf(w[s], ld_cluster_f32(cluster_addr(row + 64, s)), l);
+            l = fmaf(w[s], ld_cluster_f32(cluster_addr(row + 64, my.first + s)), l);
           }
         }
         if (!(l > 0.f)) flag_status(a.status, kStatusBadRow);
         const float inv = l > 0.f ? 1.0f / l : 0.f;
-        const int s0 = (int)cluster_rank();
         uint2* dst = reinterpret_cast<uint2*>(static_cast<uint16_t*>(a.O) + ((int64_t)token * a.H + h) * 64);
-        for (int c = 16 * s0 / a.split; c < 16 * (s0 + 1) / a.split; ++c) {  // four channels each
+        for (int c = 16 * my.s / my.parts; c < 16 * (my.s + 1) / my.parts; ++c) {  // four channels each
           float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
           for (int s = 0; s < kMaxSplit; ++s)
-            if (s < a.split) {
-              const float4 v = ld_cluster_f32x4(cluster_addr(row + 4 * c, s));
+            if (s < my.parts) {
+              const float4 v = ld_cluster_f32x4(cluster_addr(row + 4 * c, my.first + s));
               o.x = fmaf(w[s], v.x, o.x);
               o.y = fmaf(w[s], v.y, o.y);
               o.z = fmaf(w[s], v.z, o.z);
@@ -814,16 +829,40 @@ static int sm_count() {
 
 int attn_num_pairs(const Shape& s) { return (s.nb + 1) / 2; }
 
-// CTAs per item of a forward's attention: with fewer items than half the CTA slots (two per
-// SM), as many as fit, up to 4.  Only the forward on the 64-token grid, whose output is not
-// tied bit for bit to ress_sparse_attn's (a share has its own reference maxima).  Lists below
-// 16 blocks gain nothing.  The whole layer with 1 / 2 / 3 / 4 CTAs per item: 2 views (88 items)
+// CTAs per item of a small forward's attention.  Where all items run at once, the longest one
+// sets the kernel's time: an item with dense query blocks walks all nb key blocks, a sparse one
+// about 1.45 times its budget (the union of two kept lists) and the always-kept blocks.  Of the
+// ways to share them that fit into one wave (two CTAs per SM), the one whose longest share is
+// shortest, if it is at least four tiles shorter than whole items.  Only the forward on the
+// 64-token grid, whose output is not tied bit for bit to ress_sparse_attn's (a share has its own
+// reference maxima).  The whole layer with 1 / 2 / 3 / 4 CTAs for every item: 2 views (88 items)
 // 89.8 / 85.7 / 85.3 / 100.8 us; 5,003 tokens x 3 heads (120 items, dense ones of 79 tiles) 106.7 /
-// 95.6 / 104.5 / 108.9; 8 views (1,376 items) 309.9 and, with two, 391.5: what does not fit into
-// one wave loses.
-int attn_split(const Shape& s) {
-  if (s.qb != kBlock || s.nb < 16) return 1;
-  return max(1, min(kMaxSplit, 2 * sm_count() / (s.H * attn_num_pairs(s))));
+// 95.6 / 104.5 / 108.9, 90.6 with 4 for the dense ones and 2 for the others; 8 views (1,376 items) 309.9 and, with two,
+// 391.5: what does not fit into one wave loses.
+AttnSplit attn_split(const Shape& s, const int32_t* c_h) {
+  AttnSplit best{1, 1};
+  if (s.qb != kBlock) return best;
+  const int npairs = attn_num_pairs(s), nd = s.H * (npairs - s.ncand / 2);
+  const int ns = s.H * npairs - nd, slots = 2 * sm_count();
+  if (nd + ns > slots) return best;
+  int c = 0;
+  for (int h = 0; h < s.H; ++h) c = max(c, c_h[h]);
+  const int sparse = min(s.nb, 29 * c / 20 + s.nb - s.ncand);
+  auto longest = [&](int split, int share) {
+    return max(nd ? (s.nb + split - 1) / split : 0, ns ? (sparse + share - 1) / share : 0);
+  };
+  int len = longest(1, 1) - 3;
+  for (int split = 2; split <= kMaxSplit; ++split)
+    for (int share = 1; share <= split; ++share) {
+      if (split % share) continue;
+      const int per = split / share;  // sparse items per cluster
+      if (split * (nd + (ns + per - 1) / per) > slots) continue;
+      if (longest(split, share) < len) {
+        len = longest(split, share);
+        best = AttnSplit{split, share};
+      }
+    }
+  return best;
 }
 
 cudaError_t launch_attn_pairs(const AttnArgs& x, cudaStream_t st) {
@@ -868,13 +907,17 @@ cudaError_t launch_attn_range(const AttnArgs& x, int p0, int p1, int slot, bool 
   p.status = x.status;
   p.counter = x.counter + slot;
   const size_t smem = sizeof(AttnSmem) + 1024;
-  p.split = x.split;
-  const bool split = x.split > 1;
+  p.split = x.split.split;
+  p.share = x.split.share;
+  const bool split = p.split > 1;
   auto kern = x.out_f32 ? k_attn<true, false> : split ? k_attn<false, true> : k_attn<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  if (split)
-    return launch_with(kern, items * x.split, kAttnThreads, smem, st, overlap, x.split, tq, tk, tv, p);
+  if (split) {
+    const int nd = s.H * max(0, p1 - max(p0, p.nsparse)), per = p.split / p.share;
+    const int clusters = nd + (items - nd + per - 1) / per;
+    return launch_with(kern, clusters * p.split, kAttnThreads, smem, st, overlap, p.split, tq, tk, tv, p);
+  }
   const int grid = min(items, 2 * sm_count());
   return launch_pdl(kern, grid, kAttnThreads, smem, st, overlap, tq, tk, tv, p);
 }

@@ -353,15 +353,15 @@ static ress::AttnArgs attn_args(const ress::Shape& s, const ress_ws_layout& L,
   a.scratch_cap = (int64_t)s.H * s.nq * s.ld;  // entries of the t array
   a.prow = nullptr;  // adjacent query blocks; a forward sets its pairing table and its split
   a.npaired = 0;
-  a.split = 1;
+  a.split = ress::AttnSplit{1, 1};
   return a;
 }
 
 // The attention of a forward uses the item table its CSR step wrote (ReSS, no variant), and
 // several CTAs per item where the layer is small.
 static void use_forward_pairing(ress::AttnArgs* a, const ress::Shape& s, const ress_ws_layout& L,
-                                void* ws) {
-  a->split = ress::attn_split(s);
+                                const int32_t* c_h, void* ws) {
+  a->split = ress::attn_split(s, c_h);
   if (ress::pairing_active(s, ress::Variant{0, 0, 0ull, 0.0f})) {
     a->prow = reinterpret_cast<const int32_t*>(static_cast<char*>(ws) + L.prow);
     a->npaired = ress::paired_items(s);
@@ -426,7 +426,7 @@ int ress_forward(const ress_dims* d, const uint16_t* Q, const uint16_t* K, const
                         J_best, nullptr, true, stream)))
     return e;
   ress::AttnArgs a = attn_args(s, L, Q, K, V, row_ptr, col_idx, col_capacity, O, false, ws);
-  use_forward_pairing(&a, s, L, ws);
+  use_forward_pairing(&a, s, L, c_h, ws);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t ce = ress::launch_attn_range(a, 0, ress::attn_num_pairs(s), 0, true, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "ress_forward attention");
@@ -478,7 +478,7 @@ int ress_forward_host(const ress_dims* d, const uint16_t* Q_host, const uint16_t
   if ((e = check_ws(s, ws, ws_bytes, &L))) return e;
   ress::AttnArgs a =
       attn_args(s, L, Q_dev, K_dev, V_dev, row_ptr, col_idx, col_capacity, O_dev, false, ws);
-  use_forward_pairing(&a, s, L, ws);
+  use_forward_pairing(&a, s, L, c_h, ws);
   std::lock_guard<std::mutex> lock(g_overlap_mu);
   OverlapStreams* o = nullptr;
   cudaError_t ce = overlap_streams(&o);
@@ -696,7 +696,7 @@ extern "C" int ress_sparse_attn_noalloc(const ress_dims* d, const uint16_t* Q, c
   a.scratch_cap = list_entries;
   a.prow = nullptr;  // items of adjacent query blocks
   a.npaired = 0;
-  a.split = 1;
+  a.split = ress::AttnSplit{1, 1};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t ce = ress::launch_sparse_attn(a, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "ress_sparse_attn_noalloc");

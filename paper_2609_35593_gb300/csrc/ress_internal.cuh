@@ -233,6 +233,12 @@ bool pairing_active(const Shape& s, const Variant& v);
 int paired_items(const Shape& s);
 cudaError_t launch_pairing(const SelectArgs& a, int32_t* prow, cudaStream_t st);
 
+// How a forward's attention shares its items (attn_split, k_attn.cu): clusters of `split` CTAs, all
+// of them on one item with dense query blocks, `share` of them on each sparse item; 1: whole items.
+struct AttnSplit {
+  int split, share;
+};
+
 struct AttnArgs {
   Shape s;
   const uint16_t *Q, *K, *V;
@@ -247,7 +253,7 @@ struct AttnArgs {
   int64_t scratch_cap;
   const int32_t* prow;  // item table of a paired forward (items p < npaired), or NULL
   int npaired;
-  int split;            // CTAs per item (attn_split; bf16 output only)
+  AttnSplit split;      // (bf16 output only)
 };
 cudaError_t launch_sparse_attn(const AttnArgs& a, cudaStream_t st);
 // The two halves of launch_sparse_attn, for callers that split the attention: the union
@@ -257,7 +263,7 @@ cudaError_t launch_sparse_attn(const AttnArgs& a, cudaStream_t st);
 // 128-token block on the paper's grid.
 constexpr int kAttnCounterSlots = 16;  // uint32 counters in the workspace's 64-byte slot
 int attn_num_pairs(const Shape& s);
-int attn_split(const Shape& s);  // CTAs per item of a forward's attention (k_attn.cu)
+AttnSplit attn_split(const Shape& s, const int32_t* c_h);
 cudaError_t launch_attn_pairs(const AttnArgs& a, cudaStream_t st);
 cudaError_t launch_attn_range(const AttnArgs& a, int p0, int p1, int slot, bool overlap,
                               cudaStream_t st);

@@ -1,7 +1,8 @@
-"""Forwards of small layers, whose attention items are shared by 2 to 4 CTAs each: output
-against the oracle on every row, and the host-buffer forward's bits.  The item counts put the
-layers on each side of the lines between 1, 2, 3 and 4 CTAs per item on 152 SMs; budgets of one
-block leave some CTAs without entries."""
+"""Forwards of small layers, whose attention items are shared by up to 4 CTAs each, dense ones by
+more than sparse ones where that shortens the longest share: output against the oracle on every
+row, and the host-buffer forward's bits.  The item counts put the layers on each side of the
+lines between the ways to share on 152 SMs; budgets of one block leave some CTAs without
+entries."""
 import pytest
 
 import synth
@@ -18,7 +19,9 @@ pytestmark = pytest.mark.gpu
     (64 * 50 + 30, 3, 35, 9),  # 78 items: 3 CTAs each; two dense blocks
     (64 * 38, 4, 0, 38),       # 76 items: 4 CTAs each, nothing dropped
     (64 * 100 - 7, 3, 0, 2),   # 150 items: 2 CTAs each
-    (64 * 153, 2, 10, 12),     # 154 items: one CTA each
+    (64 * 77 + 38, 3, 37, 31),  # 117 items: 4 CTAs for the dense ones, 2 for the others
+    (64 * 130, 3, 70, 7),      # 195 items: 2 CTAs for the dense ones, one for the others
+    (64 * 205, 3, 10, 12),     # 309 items: more than one wave, whole items
 ])
 def test_split_items(N, H, ns, c):
     inp = synth.make_random_layer(N, H, 64 * H, seed=N + H)
