@@ -1556,79 +1556,130 @@ __global__ void k_csr(SelPtrs p, Budgets bud, CsrBases cb, int H, CsrOut o) {
     P = min(__reduce_add_sync(kFull, nA), __reduce_add_sync(kFull, nB));
   }
   ptx::pdl_trigger();
-  // Lane l owns word w0 + l of each row: warp scans of the lanes' counts give every word's
-  // first list positions, then each lane writes the blocks of its own word.
   int posU = 0, cA = 0, cB = 0, cR = 0;
-  for (int w0 = 0; w0 < p.words; w0 += 32) {
-    const int w = w0 + lane;
-    uint32_t keep[2] = {0u, 0u};
+  // Two ways to write the lists.  By words: lane b holds block 32 w + b of the word at hand, and
+  // each list's entries of the word leave as one store; about 40 instructions a word.  By lanes:
+  // lane l lists the blocks of word w0 + l by itself, as many steps (of about 36 instructions) as
+  // the fullest of 32 words keeps blocks, and scans for the positions; for sparse lists over
+  // many words.  k_csr by lanes / by words: 2 views (half kept, 2 words) 10.5 / 6.0 us, 64 views
+  // half kept (43 words) 85 / 42, 32 views a tenth kept (22 words) 20 / 26, 100 views (68 words)
+  // 85 / 154; the line estimates the fullest word as twice the mean and 4.
+  const int rounds = (p.words + 31) / 32, mean = max(expect[0], expect[1]) / p.words;
+  if (10 * p.words <= rounds * (9 * min(32, 2 * mean + 4) + 38)) {
+    const uint32_t below = (1u << lane) - 1u;
+    for (int w0 = 0; w0 < p.words; w0 += 32) {
+      const int w = w0 + lane;
+      uint32_t keep[2] = {0u, 0u};
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      if (r < nr && w < p.words) {
-        const uint32_t dm = drop_word(r, w);
-        if (o.drop_mask) o.drop_mask[ri[r] * p.words + w] = dm;
-        keep[r] = ~dm & valid_bits(w, p.nb);
+      for (int r = 0; r < 2; ++r) {
+        if (r < nr && w < p.words) {
+          const uint32_t dm = drop_word(r, w);
+          if (o.drop_mask) o.drop_mask[ri[r] * p.words + w] = dm;
+          keep[r] = ~dm & valid_bits(w, p.nb);
+        }
+      }
+      const int cnt = min(32, p.words - w0);
+      for (int k = 0; k < cnt; ++k) {
+        const uint32_t ka = __shfl_sync(kFull, keep[0], k), kb0 = __shfl_sync(kFull, keep[1], k);
+        const int j = 32 * (w0 + k) + lane;
+        const bool inA = (ka >> lane) & 1u, inB = (kb0 >> lane) & 1u;
+        const int pA = pos[0] + __popc(ka & below), pB = pos[1] + __popc(kb0 & below);
+        if (inA && pA < expect[0] && off[0] + pA < o.cap) o.col_idx[off[0] + pA] = j;
+        if (inB && pB < expect[1] && off[1] + pB < o.cap) o.col_idx[off[1] + pB] = j;
+        pos[0] += __popc(ka);
+        pos[1] += __popc(kb0);
+        if (o.plist) {
+          // a 128-token query block keeps its list for both 64-row halves of the tile
+          const uint32_t kb = rpi == 1 ? ka : kb0;
+          const uint32_t oa = ka & ~kb, ob = kb & ~ka;  // one-sided
+          const int rA = cA + __popc(oa & below), rB = cB + __popc(ob & below);
+          const bool altA = ((oa >> lane) & 1u) && rA < P, altB = ((ob >> lane) & 1u) && rB < P;
+          const bool rest = (((ka | kb) >> lane) & 1u) && !altA && !altB;
+          const uint32_t restw = __ballot_sync(kFull, rest);
+          const int at = altA ? 2 * rA : altB ? 2 * rB + 1 : 2 * P + cR + __popc(restw & below);
+          const int e = j | (int)(inA ? 1u << 16 : 0u) | (int)(((kb >> lane) & 1u) << 17);
+          if ((altA || altB || rest) && uoff + at < o.plist_cap) o.plist[uoff + at] = e;
+          cA += __popc(oa);
+          cB += __popc(ob);
+          cR += __popc(restw);
+          posU += __popc(ka | kb);
+        }
       }
     }
-    // a 128-token query block keeps its list for both 64-row halves of the tile
-    const uint32_t kb = rpi == 1 ? keep[0] : keep[1];
-    const uint32_t un = o.plist ? (keep[0] | kb) : 0u;
-    const uint32_t oa = P ? keep[0] & ~kb : 0u, ob = P ? kb & ~keep[0] : 0u;  // one-sided
-    const int cAB = __popc(keep[0]) | (__popc(keep[1]) << 16), cU = __popc(un);
-    const int cO = __popc(oa) | (__popc(ob) << 16);
-    int iAB = cAB, iU = cU, iO = cO;
+  } else {
+    // Lane l owns word w0 + l of each row: warp scans of the lanes' counts give every word's
+    // first list positions, then each lane writes the blocks of its own word.
+    for (int w0 = 0; w0 < p.words; w0 += 32) {
+      const int w = w0 + lane;
+      uint32_t keep[2] = {0u, 0u};
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int yAB = __shfl_up_sync(kFull, iAB, d), yU = __shfl_up_sync(kFull, iU, d);
-      const int yO = __shfl_up_sync(kFull, iO, d);
-      if (lane >= d) {
-        iAB += yAB;
-        iU += yU;
-        iO += yO;
+      for (int r = 0; r < 2; ++r) {
+        if (r < nr && w < p.words) {
+          const uint32_t dm = drop_word(r, w);
+          if (o.drop_mask) o.drop_mask[ri[r] * p.words + w] = dm;
+          keep[r] = ~dm & valid_bits(w, p.nb);
+        }
       }
-    }
-    const int tAB = __shfl_sync(kFull, iAB, 31), tU = __shfl_sync(kFull, iU, 31);
-    const int tO = __shfl_sync(kFull, iO, 31);
-    csr_write_word(o, keep[0], w, pos[0] + ((iAB - cAB) & 0xffff), expect[0], off[0]);
-    csr_write_word(o, keep[1], w, pos[1] + ((iAB - cAB) >> 16), expect[1], off[1]);
-    if (o.plist) {
-      // ranks of this word's first one-sided blocks; its lowest mA (mB) of them alternate
-      const int gA = cA + ((iO - cO) & 0xffff), gB = cB + ((iO - cO) >> 16);
-      const int mA = min(max(P - gA, 0), __popc(oa)), mB = min(max(P - gB, 0), __popc(ob));
-      const int cRest = cU - mA - mB;
-      int iR = cRest;
+      // a 128-token query block keeps its list for both 64-row halves of the tile
+      const uint32_t kb = rpi == 1 ? keep[0] : keep[1];
+      const uint32_t un = o.plist ? (keep[0] | kb) : 0u;
+      const uint32_t oa = P ? keep[0] & ~kb : 0u, ob = P ? kb & ~keep[0] : 0u;  // one-sided
+      const int cAB = __popc(keep[0]) | (__popc(keep[1]) << 16), cU = __popc(un);
+      const int cO = __popc(oa) | (__popc(ob) << 16);
+      int iAB = cAB, iU = cU, iO = cO;
 #pragma unroll
       for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(kFull, iR, d);
-        if (lane >= d) iR += y;
-      }
-      int kA = 0, kB = 0, at = 2 * P + cR + iR - cRest;
-      for (uint32_t bits = un; bits; bits &= bits - 1u) {
-        const int b = __ffs(bits) - 1;
-        const int j = w * 32 + b;
-        int64_t dst;
-        int e;
-        if ((oa >> b) & 1u) {
-          dst = kA < mA ? 2 * (gA + kA) : at++;
-          e = j | (1 << 16);
-          ++kA;
-        } else if ((ob >> b) & 1u) {
-          dst = kB < mB ? 2 * (gB + kB) + 1 : at++;
-          e = j | (2 << 16);
-          ++kB;
-        } else {
-          dst = at++;
-          e = j | (((int)((keep[0] >> b) & 1u) | (int)(((kb >> b) & 1u) << 1)) << 16);
+        const int yAB = __shfl_up_sync(kFull, iAB, d), yU = __shfl_up_sync(kFull, iU, d);
+        const int yO = __shfl_up_sync(kFull, iO, d);
+        if (lane >= d) {
+          iAB += yAB;
+          iU += yU;
+          iO += yO;
         }
-        if (uoff + dst < o.plist_cap) o.plist[uoff + dst] = e;
       }
-      cR += __shfl_sync(kFull, iR, 31);
+      const int tAB = __shfl_sync(kFull, iAB, 31), tU = __shfl_sync(kFull, iU, 31);
+      const int tO = __shfl_sync(kFull, iO, 31);
+      csr_write_word(o, keep[0], w, pos[0] + ((iAB - cAB) & 0xffff), expect[0], off[0]);
+      csr_write_word(o, keep[1], w, pos[1] + ((iAB - cAB) >> 16), expect[1], off[1]);
+      if (o.plist) {
+        // ranks of this word's first one-sided blocks; its lowest mA (mB) of them alternate
+        const int gA = cA + ((iO - cO) & 0xffff), gB = cB + ((iO - cO) >> 16);
+        const int mA = min(max(P - gA, 0), __popc(oa)), mB = min(max(P - gB, 0), __popc(ob));
+        const int cRest = cU - mA - mB;
+        int iR = cRest;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const int y = __shfl_up_sync(kFull, iR, d);
+          if (lane >= d) iR += y;
+        }
+        int kA = 0, kB = 0, at = 2 * P + cR + iR - cRest;
+        for (uint32_t bits = un; bits; bits &= bits - 1u) {
+          const int b = __ffs(bits) - 1;
+          const int j = w * 32 + b;
+          int64_t dst;
+          int e;
+          if ((oa >> b) & 1u) {
+            dst = kA < mA ? 2 * (gA + kA) : at++;
+            e = j | (1 << 16);
+            ++kA;
+          } else if ((ob >> b) & 1u) {
+            dst = kB < mB ? 2 * (gB + kB) + 1 : at++;
+            e = j | (2 << 16);
+            ++kB;
+          } else {
+            dst = at++;
+            e = j | (((int)((keep[0] >> b) & 1u) | (int)(((kb >> b) & 1u) << 1)) << 16);
+          }
+          if (uoff + dst < o.plist_cap) o.plist[uoff + dst] = e;
+        }
+        cR += __shfl_sync(kFull, iR, 31);
+      }
+      pos[0] += tAB & 0xffff;
+      pos[1] += tAB >> 16;
+      posU += tU;
+      cA += tO & 0xffff;
+      cB += tO >> 16;
     }
-    pos[0] += tAB & 0xffff;
-    pos[1] += tAB >> 16;
-    posU += tU;
-    cA += tO & 0xffff;
-    cB += tO >> 16;
   }
   if (lane == 0) {
     for (int r = 0; r < nr; ++r) {
