@@ -310,18 +310,17 @@ __device__ __forceinline__ uint32_t order_key(float x) {
 // the m largest keys, ties to the lower block index (the order the oracle uses).  Result:
 // the chosen blocks' bits in sel[words].
 //
-// 1. lower bound: the m-th largest value among every lane's local top-ceil(m/32) keys is
-//    <= the m-th largest key overall (those 32 ceil(m/32) values include m entries);
+// 1. lower bound: the m-th largest of the lanes' largest keys is <= the m-th largest key overall;
 // 2. survivors: the keys >= that bound (usually about 1.5 m of them) are compacted, in block
 //    order, into a short list;
 // 3. the m-th largest survivor T is found by a radix select over the survivors (8-bit
 //    digits; select_radix) and the survivors > T plus the lowest-index ones == T are chosen.
-// When m needs more than kTopK candidates per lane, warp_topm_large selects on all keys; when
-// too many keys tie at the bound, step 3 runs bit by bit on all keys (select_exact: same
-// result, slower).  The restoration rounds use warp_topm_pair (m <= 64) or warp_topm_large,
-// which select on both sides of the drop set at once.
+// That is for small m; larger ones take warp_topm_large, on all keys (keeping ceil(m / 32) keys per
+// lane for the bound was the slower way: 32 views, m = 68, 47.7 against 44.8 us for the scoring
+// row kernel).  When too many keys tie at the bound, step 3 runs bit by bit on all keys
+// (select_exact: same result, slower).  The restoration rounds use warp_topm_pair (m <= 64) or
+// warp_topm_large, which select on both sides of the drop set at once.
 // ------------------------------------------------------------------------------------
-constexpr int kTopK = 4;          // lane-local candidates: fast path for m <= 128
 constexpr int kSurvivors = 256;   // capacity of the survivor list
 
 __device__ __forceinline__ bool takes_part(const uint32_t* member, bool want, int j) {
@@ -510,91 +509,115 @@ __device__ void select_radix(const uint32_t* keys, const uint16_t* idx, int n, i
 // largest keys among the blocks of the drop set Dw into selD and the m largest among the
 // other candidates into selB at once (every key belongs to one side, so both sides share each
 // pass); otherwise the m largest of all keys into selD.  Ties go to the lower index; a side
-// with fewer than m blocks is taken whole.  Three passes over the keys, 32 consecutive blocks
-// at a time so that a mask word is one ballot: counts by the top byte, counts by the second
-// byte of the keys that share the m-th key's top byte, then the choice; the few keys that
-// share its upper 16 bits are ranked among themselves (a side with more than 128 of those,
-// heavy ties, takes select_exact).  A bit-by-bit search over the keys, which this replaces
-// for m > 64 (rounds) and m > 128 (initial selection), makes up to 32 passes per side: at 64
-// views and half the blocks dropped (m = 171, 1369 keys) the round kernel took 774 us with it
-// and 313 us with this.
+// with fewer than m blocks is taken whole.  topD, topB: this lane's largest key on each side.
+//
+// Keys are counted by their distance below their side's largest key, in steps of 2^19 (float
+// keys: 1/16 octave, so the 256 counters reach 16 octaves down), so that the counted keys spread
+// over the counters and those too far down to matter touch none: with the counters on the top
+// byte of the key (the exponent, nearly the same for all), half of the shared-memory pipe's
+// cycles went to lanes adding to one counter in turn.  Three passes, 32 consecutive blocks at a
+// time so that a mask word is one ballot: counts by the distance's upper part, counts by its
+// next 8 bits within the m-th key's step, then the choice; the few keys that share those bits too
+// are ranked among themselves (a side with more than 128 of them, heavy ties, takes
+// select_exact).  Where a side's m-th key is further down, both sides count by the key's own top
+// two bytes instead.  A bit-by-bit search over the keys makes up to 32 passes per side: at 64 views
+// and half the blocks dropped (m = 171, 1369 keys) the round kernel took 774 us with it, 313
+// counting by bytes and 305 so; the initial selection (c = 684) 492, 411 and 339; at 100 views
+// (c = 214, 2142 keys) 632, 640 and 451.
 template <bool PAIR>
 __device__ void warp_topm_large(const uint32_t* kk, int n, int m, const uint32_t* Dw,
                                 uint32_t* selD, uint32_t* selB, int words, uint32_t* sk,
-                                uint16_t* si) {
+                                uint16_t* si, uint32_t topD, uint32_t topB) {
   constexpr int kSides = PAIR ? 2 : 1;
   constexpr int kHalf = kSurvivors / 2;
   const int lane = threadIdx.x & 31;
   const uint32_t below = (1u << lane) - 1u;
-  int prefix[2] = {0, 0}, need[2] = {m, m}, cnt[2] = {0, 0};
-#pragma unroll
-  for (int pass = 0; pass < 2; ++pass) {
-    reinterpret_cast<uint4*>(sk)[lane] = make_uint4(0u, 0u, 0u, 0u);
-    if (PAIR) reinterpret_cast<uint4*>(sk)[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
-    __syncwarp();
+  uint32_t top[2] = {__reduce_max_sync(kFull, topD), PAIR ? __reduce_max_sync(kFull, topB) : 0u};
+  int shift = 19;
+  uint32_t prefix[2];  // the m-th key's distance, its bits from `shift` up
+  int need[2], cnt[2];
+#pragma unroll 1
+  for (;;) {
+    prefix[0] = prefix[1] = 0u;
+    need[0] = need[1] = m;
+    cnt[0] = cnt[1] = 0;
+    bool far = false;
+#pragma unroll 1
+    for (int pass = 0; pass < 2 && !far; ++pass, shift -= 8) {
+      reinterpret_cast<uint4*>(sk)[lane] = make_uint4(0u, 0u, 0u, 0u);
+      if (PAIR) reinterpret_cast<uint4*>(sk)[32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+      __syncwarp();
 #pragma unroll 4
-    for (int w = 0; w < words; ++w) {
-      const int x = 32 * w + lane;
-      if (x < n) {
-        const uint32_t v = kk[x];
-        const int side = PAIR ? (int)(~(Dw[w] >> lane) & 1u) : 0;  // 0: in D (or all), 1: not
-        const uint32_t d = pass == 0 ? v >> 24 : (v >> 16) & 255u;
-        if (pass == 0 || (int)(v >> 24) == (side ? prefix[1] : prefix[0]))
-          atomicAdd(&sk[128 * side + (d >> 1)], 1u << (16 * (d & 1u)));
-      }
-    }
-    __syncwarp();
-    // lane l owns digits base + 7 .. base, base = 8 (31 - l): lane 0 the highest; one scan
-    // carries both sides' counts (16 bits each; n <= 4096)
-    uint32_t c[2][4];
-    int sum = 0;
-#pragma unroll
-    for (int t = 0; t < kSides; ++t) {
-      const uint4 q = reinterpret_cast<const uint4*>(sk)[32 * t + 31 - lane];
-      c[t][0] = q.w; c[t][1] = q.z; c[t][2] = q.y; c[t][3] = q.x;
-      const uint32_t two = (q.x + q.y) + (q.z + q.w);  // no carry: at most 4096 in all
-      sum += (int)((two & 0xffffu) + (two >> 16)) << (16 * t);
-    }
-    int inc = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += y;
-    }
-    const int total = __shfl_sync(kFull, inc, 31);
-#pragma unroll
-    for (int t = 0; t < kSides; ++t) {
-      if (pass == 0) need[t] = min(need[t], (total >> (16 * t)) & 0xffff);
-      const int mine = (sum >> (16 * t)) & 0xffff;
-      const int in_t = (inc >> (16 * t)) & 0xffff, ex_t = in_t - mine;
-      const uint32_t who = __ballot_sync(kFull, ex_t < need[t] && need[t] <= in_t);
-      int found = 0;  // digit | count << 8 | keys above the digit << 20
-      if ((who >> lane) & 1u) {
-        int run = ex_t;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const int k = (int)((i & 1) ? c[t][i >> 1] & 0xffffu : c[t][i >> 1] >> 16);
-          if (found == 0 && run + k >= need[t]) found = (8 * (31 - lane) + 7 - i) | (k << 8);
-          if (found == 0) run += k;
+      for (int w = 0; w < words; ++w) {
+        const int x = 32 * w + lane;
+        if (x < n) {
+          const bool other = PAIR && !((Dw[w] >> lane) & 1u);
+          // within the step found so far: 0 .. 255 (pass 0: from the top)
+          const uint32_t d = (((other ? top[1] : top[0]) - kk[x]) >> shift) -
+                             ((other ? prefix[1] : prefix[0]) << 8);
+          if (d < 256u) atomicAdd(&sk[(other ? 128 : 0) + (d >> 1)], 1u << (16 * (d & 1u)));
         }
-        need[t] -= run;
       }
-      const int src = who ? __ffs(who) - 1 : 0;  // none: need is 0, nothing to choose
-      found = __shfl_sync(kFull, found, src);
-      need[t] = __shfl_sync(kFull, need[t], src);
-      prefix[t] = (prefix[t] << 8) | (found & 255);
-      cnt[t] = found >> 8;
-      if (!who) prefix[t] = pass == 0 ? 255 : 0xffff;
+      __syncwarp();
+      // lane l owns digits 8 l .. 8 l + 7; one scan carries both sides' counts (16 bits each;
+      // n <= 4096)
+      uint32_t c[2][4];
+      int sum = 0;
+#pragma unroll
+      for (int t = 0; t < kSides; ++t) {
+        const uint4 q = reinterpret_cast<const uint4*>(sk)[32 * t + lane];
+        c[t][0] = q.x; c[t][1] = q.y; c[t][2] = q.z; c[t][3] = q.w;
+        const uint32_t two = (q.x + q.y) + (q.z + q.w);  // no carry: at most 4096 in all
+        sum += (int)((two & 0xffffu) + (two >> 16)) << (16 * t);
+      }
+      int inc = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+      }
+      const int total = __shfl_sync(kFull, inc, 31);
+#pragma unroll
+      for (int t = 0; t < kSides; ++t) {
+        const int all = (total >> (16 * t)) & 0xffff;
+        if (pass == 0 && all < need[t]) {  // the m-th key is further down, or there is none
+          if (shift == 19) far = true;
+          need[t] = all;
+        }
+        const int mine = (sum >> (16 * t)) & 0xffff;
+        const int in_t = (inc >> (16 * t)) & 0xffff, ex_t = in_t - mine;
+        const uint32_t who = __ballot_sync(kFull, ex_t < need[t] && need[t] <= in_t);
+        int found = 0;  // digit | count << 8
+        if ((who >> lane) & 1u) {
+          int run = ex_t;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const int k = (int)((i & 1) ? c[t][i >> 1] >> 16 : c[t][i >> 1] & 0xffffu);
+            if (found == 0 && run + k >= need[t]) found = (8 * lane + i) | (k << 8);
+            if (found == 0) run += k;
+          }
+          need[t] -= run;
+        }
+        const int src = who ? __ffs(who) - 1 : 0;  // none: need is 0, nothing to choose
+        found = __shfl_sync(kFull, found, src);
+        need[t] = __shfl_sync(kFull, need[t], src);
+        prefix[t] = (prefix[t] << 8) | (uint32_t)(found & 255);
+        cnt[t] = found >> 8;
+      }
+      __syncwarp();
     }
-    __syncwarp();
+    if (!far) break;
+    top[0] = top[1] = kFull;  // by the keys' own top two bytes: every key is within reach
+    shift = 24;
   }
-  // keys above gt[side] are chosen; those whose upper half is eq[side] are listed
-  int gt[2], eq[2], listed[2] = {0, 0};
+  shift += 8;  // of the last pass
+  // keys nearer than near[side] are chosen; those at tied[side] are listed
+  int near[2], tied[2], listed[2] = {0, 0};
 #pragma unroll
   for (int t = 0; t < 2; ++t) {
     const bool all = cnt[t] == need[t] && need[t] > 0;
-    gt[t] = all ? prefix[t] - 1 : prefix[t];
-    eq[t] = (all || need[t] == 0) ? -2 : prefix[t];
+    near[t] = need[t] == 0 ? 0 : (int)prefix[t] + (all ? 1 : 0);
+    tied[t] = (all || need[t] == 0) ? -1 : (int)prefix[t];
   }
 #pragma unroll 2
   for (int w = 0; w < words; ++w) {
@@ -602,9 +625,9 @@ __device__ void warp_topm_large(const uint32_t* kk, int n, int m, const uint32_t
     const uint32_t v = x < n ? kk[x] : 0u;
     const uint32_t dw = PAIR ? Dw[w] : kFull;
     const bool inD = (dw >> lane) & 1u;
-    const int v16 = (int)(v >> 16);
-    const uint32_t pick = __ballot_sync(kFull, x < n && v16 > (PAIR && !inD ? gt[1] : gt[0]));
-    const uint32_t tie = __ballot_sync(kFull, x < n && v16 == (PAIR && !inD ? eq[1] : eq[0]));
+    const int d = (int)(((PAIR && !inD ? top[1] : top[0]) - v) >> shift);
+    const uint32_t pick = __ballot_sync(kFull, x < n && d < (PAIR && !inD ? near[1] : near[0]));
+    const uint32_t tie = __ballot_sync(kFull, x < n && d == (PAIR && !inD ? tied[1] : tied[0]));
     if (lane == 0) {
       selD[w] = pick & dw;
       if (PAIR) selB[w] = pick & ~dw;
@@ -624,7 +647,7 @@ __device__ void warp_topm_large(const uint32_t* kk, int n, int m, const uint32_t
   __syncwarp();
 #pragma unroll
   for (int t = 0; t < kSides; ++t) {
-    if (eq[t] < 0) continue;
+    if (tied[t] < 0) continue;
     uint32_t* sel = t ? selB : selD;
     const int L = listed[t];
     if (L > kHalf) {
@@ -647,49 +670,17 @@ __device__ void warp_topm_large(const uint32_t* kk, int n, int m, const uint32_t
   __syncwarp();
 }
 
-// The lower bound of step 1 with KT = ceil(m / 32) keys kept per lane: the m-th largest of
-// the lanes' KT largest keys.
-template <int KT>
-__device__ __forceinline__ uint32_t lane_topk_bound(const uint32_t* kk, int n, int m) {
-  const int lane = threadIdx.x & 31;
-  uint32_t top[KT];
-#pragma unroll
-  for (int k = 0; k < KT; ++k) top[k] = 0u;
-#pragma unroll 2
-  for (int x = lane; x < n; x += 32) {
-    uint32_t v = kk[x];
-#pragma unroll
-    for (int k = 0; k < KT; ++k) {
-      const uint32_t hi = max(top[k], v);
-      v = min(top[k], v);
-      top[k] = hi;
-    }
-  }
-  return mth_largest(top, m);
-}
-
-// Requires m <= n.  sk/si: survivor scratch (kSurvivors); hist: 256 words for select_radix on
-// the survivors.
-// LARGE: m may exceed 32 kTopK.
-template <bool LARGE>
+// The m <= 32 largest of n keys, m <= n.  sk/si: survivor scratch (kSurvivors); hist: 256 words
+// for select_radix on the survivors; top: this lane's largest key.
 __device__ void warp_topm(const uint32_t* kk, int n, int m, uint32_t* sel, int words,
-                          uint32_t* sk, uint16_t* si, uint32_t* hist) {
+                          uint32_t* sk, uint16_t* si, uint32_t* hist, uint32_t top) {
   const int lane = threadIdx.x & 31;
-  if (LARGE && m > 32 * kTopK) {
-    warp_topm_large<false>(kk, n, m, nullptr, sel, nullptr, words, sk, si);
-    return;
-  }
   for (int w = lane; w < words; w += 32) sel[w] = 0u;
   __syncwarp();
   if (m <= 0) return;
-  // 1. lane-local top-K (descending), then the lower bound
-  uint32_t bound;
-  switch ((m + 31) / 32) {
-    case 1: bound = lane_topk_bound<1>(kk, n, m); break;
-    case 2: bound = lane_topk_bound<2>(kk, n, m); break;
-    case 3: bound = lane_topk_bound<3>(kk, n, m); break;
-    default: bound = lane_topk_bound<4>(kk, n, m); break;
-  }
+  // 1. the m-th largest of the lanes' largest keys
+  const uint32_t tops[1] = {top};
+  const uint32_t bound = mth_largest(tops, m);
   // 2. survivors (>= bound), compacted in block order
   int cnt = 0;
   for (int x0 = 0; x0 < n; x0 += 32) {
@@ -780,6 +771,26 @@ __device__ bool warp_topm_pair(const uint32_t* kk, int n, int m, const uint32_t*
   const uint32_t bD = mth_of_64(top.d1, top.d2, m), bB = mth_of_64(top.b1, top.b2, m);
   constexpr int kHalf = kSurvivors / 2;
   int cntD = 0, cntB = 0;
+  if (LARGE && m > 32) {
+    // where the lists nearly always overflow: count first (100 views, m = 53: 717 us for the
+    // round without, 603 with)
+    int c = 0;
+    for (int x = 4 * lane; x < n; x += 128) {
+      const uint4 v = *reinterpret_cast<const uint4*>(kk + x);
+      const uint32_t dbits = Dw[x >> 5] >> (x & 31);
+      const uint32_t k4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool inD = (dbits >> u) & 1u;
+        if (x + u < n && k4[u] >= (inD ? bD : bB)) c += inD ? 1 : 0x10000;
+      }
+    }
+    c = __reduce_add_sync(kFull, c);
+    if ((c & 0xffff) > kHalf || (c >> 16) > kHalf) {
+      warp_topm_large<true>(kk, n, m, Dw, selD, selB, words, sk, si, top.d1, top.b1);
+      return false;
+    }
+  }
   // survivors in ascending block order, four consecutive blocks per lane and step: each
   // lane's counts on both sides (packed) go through one warp scan for the store positions
   for (int x0 = 0; x0 < n; x0 += 128) {
@@ -834,7 +845,7 @@ __device__ bool warp_topm_pair(const uint32_t* kk, int n, int m, const uint32_t*
   __syncwarp();
   const bool listed = cntD <= kHalf && cntB <= kHalf;
   if (LARGE && !listed) {
-    warp_topm_large<true>(kk, n, m, Dw, selD, selB, words, sk, si);
+    warp_topm_large<true>(kk, n, m, Dw, selD, selB, words, sk, si, top.d1, top.b1);
     return false;
   }
   // one copy of each selection for both sides: the kernel waits on instruction fetch (108 KB of
@@ -1106,10 +1117,10 @@ __device__ void cdf_extend(const uint32_t* kk, const float* __restrict__ Prow, u
 // 24 bits of SplitMix64 at seed + (h 4096 + i) 4096 + j; the full sign flip keeps the
 // smallest keys (complemented keys, ties still to the lower index).
 // KEY: the key variant (v.key), a template parameter so that the per-block key has no branch.
-// LARGE: some head's budget exceeds 32 kTopK (the selection on all keys is compiled in; it
-// takes more registers, and rows that long leave room for fewer warps anyway).
+// LARGE: selection by warp_topm_large, for any budget (launch_score draws the line); else by
+// warp_topm.
 template <int KEY, bool LARGE>
-__global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(SelPtrs p, Budgets bud,
+__global__ void __launch_bounds__(32 * kRowWarps, 9) k_score_rows(SelPtrs p, Budgets bud,
                                                                   Variant v) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ptx::pdl_wait();
@@ -1128,6 +1139,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(Se
   uint32_t* sel = sk + kSurvivors + kSurvivors / 2;
   // radix counters: in the spent key area, or after the mask when the CDF rule needs the keys
   uint32_t* hist = v.cdf > 0.f ? sel + (p.words + 3) / 4 * 4 : kk;
+  uint32_t top = 0u;  // this lane's largest key
   row_keys(p.ncand, kk, [&](int j, uint32_t (&k4)[4]) {
     const float4 P4 = *reinterpret_cast<const float4*>(Prow + j);
     const float4 q4 = *reinterpret_cast<const float4*>(qrow + j);
@@ -1144,8 +1156,14 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 9) k_score_rows(Se
                                                  4096ull + (unsigned long long)(j + u)) >> 40) + 1u;
       k4[u] = (v.direction == 2) ? ~key : key;
     }
-  }, [](int, const uint32_t (&)[4]) {});
-  warp_topm<LARGE>(kk, p.ncand, bud.c[h], sel, p.words, sk, si, hist);  // sel = kept
+  }, [&](int, const uint32_t (&k4)[4]) {
+    top = max(max(top, max(k4[0], k4[1])), max(k4[2], k4[3]));
+  });
+  // sel = kept
+  if (LARGE)
+    warp_topm_large<false>(kk, p.ncand, bud.c[h], nullptr, sel, nullptr, p.words, sk, si, top, 0u);
+  else
+    warp_topm(kk, p.ncand, bud.c[h], sel, p.words, sk, si, hist, top);
   ptx::pdl_trigger();
   // drop set D0 = candidates not kept
   for (int w = lane; w < p.words; w += 32) sel[w] = valid_bits(w, p.ncand) & ~sel[w];
@@ -1245,7 +1263,7 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 10) k_round_rows(S
   if (!LARGE || m <= 64) {
     listed = warp_topm_pair<LARGE>(kk, p.ncand, m, Dw, top, Rw, Xw, p.words, sk, si, lst);
   } else {
-    warp_topm_large<true>(kk, p.ncand, m, Dw, Rw, Xw, p.words, sk, si);
+    warp_topm_large<true>(kk, p.ncand, m, Dw, Rw, Xw, p.words, sk, si, top.d1, top.b1);
   }
   if (round == 0) {
     // both selections took m blocks from their side only if the drop set holds that many on
@@ -1764,7 +1782,9 @@ cudaError_t launch_score(const SelectArgs& a, cudaStream_t st) {
       (size_t)kRowWarps * warp_scratch_words(s.ld, score_mask_words(s.words, a.v.cdf > 0.f)) * 4;
   int cmax = 0;
   for (int h = 0; h < s.H; ++h) cmax = max(cmax, a.c[h]);
-  const bool large = cmax > 32 * kTopK;
+  // scoring stage by survivor lists / on all keys: 32 views, c = 7 142.3 / 148.9 us, c = 14 148.4 /
+  // 150.3; 8 views, c = 9 65.0 / 65.8; 2 views, 42 keys, c = 4 30.6 / 27.9, c = 21 31.2 / 28.5
+  const bool large = cmax > 16 || s.ncand <= 64;
   auto kern = a.v.key == 0   ? (large ? k_score_rows<0, true> : k_score_rows<0, false>)
               : a.v.key == 1 ? (large ? k_score_rows<1, true> : k_score_rows<1, false>)
                              : (large ? k_score_rows<2, true> : k_score_rows<2, false>);

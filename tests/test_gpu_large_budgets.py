@@ -40,3 +40,20 @@ def test_equal_keys_beyond_the_tie_list(c):
     want = np.ones(layer.nb, dtype=bool)
     want[:c] = False
     assert (layer.drop_sets()[:, :layer.nqc] == want).all()
+
+
+@pytest.mark.parametrize("c,R", [(200, 0), (290, 0)])
+def test_keys_over_many_octaves(c, R):
+    """Keys scaled so that the pooled probabilities of a row span far more than the 16 octaves
+    below the largest key that the selection counts first: the c-th key lies beyond them."""
+    N, H = 64 * 300, 1
+    inp = synth.make_random_layer(N, H, 64 * H, seed=300 + c)
+    inp["K"] = synth.bf16_bits(synth.bf16_to_f32(inp["K"]) * np.float32(24.0))
+    layer = G.Layer(inp, 0, [c], R, variant=O.Variant(key="probability"), q_block=128).run(attention=False)
+    P = layer.ws("P", shape=(H, layer.nq, layer.buf.layout.ld))[0, :layer.nqc, :layer.ncand]
+    cth = np.sort(P, axis=1)[:, -c]
+    assert np.median(P.max(1) / np.maximum(cth, 1e-30)) > 2.0 ** 16
+    # the drop sets alone: a row here drops a pooled mass far below the float32 rounding of its
+    # kept mass, from which its net drift is formed, so its J (about 1e-20) has no relative accuracy
+    r = G.compare_selection(layer, layer.oracle_select())
+    assert r["mismatched"] == 0 and r["near"] <= G.NEAR_FRACTION * (r["exact"] + r["near"]) + 1, r
