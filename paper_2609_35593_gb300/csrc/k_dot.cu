@@ -15,17 +15,23 @@
 // The three dropped products are below 2^-23 of |x||w| together, the size of the fp32
 // rounding of the dot product itself.
 //
-// One CTA per 128 x 128 tile of (i, j) of one head, 128 threads:
-//   thread 0   TMA of the six 128 x 64 bf16 term tiles (128-byte swizzle) on one mbarrier;
+// One CTA per 128 x 128 tile of (i, j) of one head, two per SM, 128 threads (logits) or 256:
+//   thread 0   TMA of the six 128 x 64 bf16 term tiles (128-byte swizzle), two per mbarrier in
+//              the order the products use them;
 //   warp 0     converged MMA warp, one elected lane issues 6 x 4 tcgen05.mma M128 N128 K16
 //              (A = x terms, B = w terms, both K-major from shared memory) and commits;
-//   warps 0-3  epilogue: tcgen05.ld of the accumulator rows (warp w: rows 32w..32w+31),
-//              the result into shared memory (the operand tiles are free by then) as four
-//              32-column boxes in the 128-byte-swizzled layout, which thread 0 writes out
-//              with TMA bulk tensor stores (rows past nb and columns past the row stride
-//              are clipped by the copy; rows past |P| are never read).
-// Every mbarrier wait is bounded; a wait that gives up records RESS_ETIMEOUT, lets copies
-// and MMAs already issued finish (again bounded), frees TMEM and returns.
+//   all warps  epilogue: tcgen05.ld of the accumulator rows (warp w: rows 32 (w mod 4)..), the
+//              result into shared memory (the operand tiles are free by then) as boxes of 32
+//              rows x 32 columns in the 128-byte-swizzled layout, each written out by its warp
+//              with a TMA bulk tensor store as soon as it is formed (columns past the row
+//              stride and rows past the array are clipped by the copy; rows past |P| are never
+//              read).
+// What bounds it is the chain of one tile (launch, loads, MMAs, epilogue, stores: about 6 us),
+// two tiles in flight per SM.  With one barrier for all operands, four epilogue warps and one
+// store of the whole tile at the end: logits 16.8 us at 32 views, 48.5 at 64, 110 at 100, now 14.7,
+// 43.2, 98.8; drift norms 46.1 -> 42.9 and 101 -> 94.5; gains 15.0, 42.8 and 96 either way.
+// Every mbarrier wait is bounded; a wait that gives up records RESS_ETIMEOUT, lets copies and
+// MMAs already issued finish (again bounded), frees TMEM and returns.
 
 #include <cudaTypedefs.h>
 
@@ -37,7 +43,6 @@ using namespace ptx;
 
 namespace {
 
-constexpr int kDotThreads = 128;
 constexpr int kDotTile = 128;                     // rows i and blocks j per CTA
 constexpr uint32_t kTermBytes = kDotTile * 128;   // 128 x 64 bf16
 constexpr uint32_t kDotCols = 128;                // TMEM columns: one fp32 128 x 128 tile
@@ -45,13 +50,17 @@ constexpr uint64_t kDotWaitNs = 2000000000ull;    // 2 s per wait
 constexpr uint64_t kDotDrainNs = 200000000ull;    // 0.2 s to drain after an abort
 
 enum DotMode { kDotGain = 0, kDotLogit = 1, kDotDist = 2 };
+// Epilogue warps: four, or eight (two per 32 rows, a half of the columns each) where no sum runs
+// along the row.
+template <int MODE>
+constexpr int kDotThreads = MODE == kDotLogit ? 128 : 256;
 constexpr float kLogitScale = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
 
 struct __align__(1024) DotSmem {
   uint8_t A[3][kTermBytes];  // row-vector terms (hi, mid, lo) of rows i0 .. i0 + 127
   uint8_t B[3][kTermBytes];  // block-vector terms of blocks j0 .. j0 + 127
   float bcol[kDotTile];      // drift norms: ||z~_j||^2 of the tile's blocks
-  uint64_t full, done;
+  uint64_t full[3], done;  // operand terms by pairs, in the order the products need them
   uint32_t tmem_base;
   int abort;
 };
@@ -85,7 +94,7 @@ __device__ __forceinline__ bool dot_wait(uint64_t* bar, uint32_t parity, volatil
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(kDotThreads)
+__global__ void __launch_bounds__(kDotThreads<MODE>)
     k_dot(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const __grid_constant__ CUtensorMap tmOut, const DotParams p) {
   const int h = blockIdx.z, i0 = blockIdx.y * kDotTile, j0 = blockIdx.x * kDotTile;
@@ -100,7 +109,7 @@ __global__ void __launch_bounds__(kDotThreads)
   volatile int* abort = &S.abort;
 
   if (threadIdx.x == 0) {
-    mbar_init(&S.full, 1);
+    for (int t = 0; t < 3; ++t) mbar_init(&S.full[t], 1);
     mbar_init(&S.done, 1);
     S.abort = 0;
     fence_barrier_init();
@@ -114,8 +123,8 @@ __global__ void __launch_bounds__(kDotThreads)
   tc_fence_after();
   pdl_wait();
   if (MODE == kDotDist) {
-    const int j = j0 + (int)threadIdx.x;  // kDotThreads == kDotTile
-    S.bcol[threadIdx.x] = j < p.nb ? p.b[(int64_t)h * p.nb + j] : 0.f;
+    const int j = j0 + (int)threadIdx.x;
+    if (threadIdx.x < kDotTile) S.bcol[threadIdx.x] = j < p.nb ? p.b[(int64_t)h * p.nb + j] : 0.f;
     __syncthreads();
   }
   const uint32_t tmem = S.tmem_base;
@@ -123,11 +132,13 @@ __global__ void __launch_bounds__(kDotThreads)
   bool issued = false;  // warp 0: MMAs went out (their completion must be awaited)
   if (warp == 0) {
     if (lane == 0) {
-      mbar_arrive_expect_tx(&S.full, 6 * kTermBytes);
+      // (mid, mid), (hi, lo), (lo, hi): the first products start while the others' terms land
 #pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        tma_load_4d(S.A[s], &tmA, &S.full, 0, i0, h, s);
-        tma_load_4d(S.B[s], &tmB, &S.full, 0, j0, h, s);
+      for (int t = 0; t < 3; ++t) {
+        const int ta = (kTermA >> (4 * t)) & 0xF, tb = (kTermB >> (4 * t)) & 0xF;
+        mbar_arrive_expect_tx(&S.full[t], 2 * kTermBytes);
+        tma_load_4d(S.A[ta], &tmA, &S.full[t], 0, i0, h, ta);
+        tma_load_4d(S.B[tb], &tmB, &S.full[t], 0, j0, h, tb);
       }
     }
     __syncwarp();
@@ -137,30 +148,37 @@ __global__ void __launch_bounds__(kDotThreads)
         flag_status(p.status, kStatusBadRow);
         *abort = 1;
       }
-    } else if (dot_wait(&S.full, 0, abort, kDotWaitNs)) {
-      tc_fence_after();
+    } else {
       const uint32_t idesc = idesc_bf16_f32(kDotTile, kDotTile, false);
-      if (leader) {
+      bool ok = true;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) {
+      for (int q = 0; q < 6; ++q) {
+        if (q < 3 && ok) {  // (the last three products use terms that have landed)
+          ok = dot_wait(&S.full[q], 0, abort, kDotWaitNs);
+          tc_fence_after();
+        }
+        if (ok && leader) {
           const uint32_t a = smem_u32(S.A[(kTermA >> (4 * q)) & 0xF]);
           const uint32_t b = smem_u32(S.B[(kTermB >> (4 * q)) & 0xF]);
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             mma_bf16_ss(tmem, sdesc_sw128(a + 32 * k), sdesc_sw128(b + 32 * k), idesc,
                         (q > 0 || k > 0) ? 1u : 0u);
+          issued = true;
         }
-        mma_commit(&S.done);
+        __syncwarp();
       }
-      __syncwarp();
-      issued = true;
-    } else if (lane == 0) {
-      flag_status(p.status, kStatusTimeout);
-      *abort = 1;
+      if (leader && issued) mma_commit(&S.done);
+      issued = __any_sync(0xffffffffu, issued);
+      if (!ok && lane == 0) {
+        flag_status(p.status, kStatusTimeout);
+        *abort = 1;
+      }
     }
-    if (!issued) {  // the copies must land before the shared memory goes away
+    if (*abort) {  // the copies must land before the shared memory goes away
       volatile int no_abort = 0;
-      if (lane == 0) mbar_wait(&S.full, 0, &no_abort, kDotDrainNs);
+      if (lane == 0)
+        for (int t = 0; t < 3; ++t) mbar_wait(&S.full[t], 0, &no_abort, kDotDrainNs);
       __syncwarp();
     }
   }
@@ -174,17 +192,20 @@ __global__ void __launch_bounds__(kDotThreads)
   }
   if (ok) {
     tc_fence_after();
-    const int r = 32 * warp + lane;  // row of the tile = TMEM lane
+    const int rw = warp & 3;            // this warp's 32 rows
+    const int r = 32 * rw + lane;       // row of the tile = TMEM lane
     const int i = i0 + r;
     const int64_t ri = (int64_t)h * p.nq + i;
     float a = 0.f;
     if (MODE != kDotLogit && i < p.nq) a = p.a[ri];
     float pm = -INFINITY, ps = 0.f;  // logits: running max and sum over the slice
-    uint8_t* stage = &S.A[0][0];     // 4 boxes of 128 rows x 32 fp32, 16 KB each
+    uint8_t* stage = &S.A[0][0];     // 4 x 4 boxes of 32 rows x 32 fp32, 4 KB each
+    constexpr int kQuarters = 512 / kDotThreads<MODE>;  // of 32 columns per warp
+    const int q0 = kQuarters * (warp >> 2);
 #pragma unroll 1
-    for (int q = 0; q < kDotTile / 32; ++q) {
+    for (int q = q0; q < q0 + kQuarters; ++q) {
       uint32_t v[32];
-      RESS_TMEM_LD32(tmem + ((uint32_t)(32 * warp) << 16) + 32 * q, v);
+      RESS_TMEM_LD32(tmem + ((uint32_t)(32 * rw) << 16) + 32 * q, v);
       float o[32];
       if (MODE == kDotGain) {
 #pragma unroll
@@ -227,18 +248,18 @@ __global__ void __launch_bounds__(kDotThreads)
       for (int k = 0; k < 8; ++k)  // 16-byte chunk k of the row goes to chunk k ^ (r mod 8)
         *reinterpret_cast<float4*>(row + ((k ^ (r & 7)) << 4)) =
             make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+      // this warp's box leaves while the next is formed
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0 && j0 + 32 * q < p.ld && i0 + 32 * rw < p.nq) {
+        tma_store_3d(&tmOut, stage + q * 16384 + rw * 4096, j0 + 32 * q, i0 + 32 * rw, h);
+        bulk_commit();
+      }
     }
     if (MODE == kDotLogit && i < p.nqc)
       p.lstat[ri * p.nslices + blockIdx.x] = make_float2(pm, ps);
-    fence_proxy_async_smem();
-  }
-  __syncthreads();
-  if (ok && threadIdx.x == 0) {
-#pragma unroll 1
-    for (int q = 0; q < kDotTile / 32; ++q)
-      if (j0 + 32 * q < p.ld) tma_store_3d(&tmOut, &S.A[0][0] + q * 16384, j0 + 32 * q, i0, h);
-    bulk_commit();
-    bulk_wait_read_all();  // the boxes are read before the shared memory goes away
+    if (lane == 0) bulk_wait_read_all();  // the boxes are read before the shared memory goes away
+    __syncwarp();
   }
   if (warp == 0 && issued && !ok) {  // MMAs still running: let them finish before the free
     volatile int no_abort = 0;
@@ -282,14 +303,14 @@ bool make_term_map(CUtensorMap* m, const void* base, int nb, int H, int rows) {
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// fp32 [H][nb][ld] viewed as {ld, nb, H}; box {32, 128, 1}, 128-byte swizzle.  Loads past
+// fp32 [H][nb][ld] viewed as {ld, nb, H}; box {32, rows, 1}, 128-byte swizzle.  Loads past
 // the edges read zeros; stores past them are dropped.
-bool make_row_map(CUtensorMap* m, void* base, int nb, int H, int ld) {
+bool make_row_map(CUtensorMap* m, void* base, int nb, int H, int ld, int rows) {
   auto fn = tensor_map_encoder();
   if (!fn) return false;
   cuuint64_t dims[3] = {(cuuint64_t)ld, (cuuint64_t)nb, (cuuint64_t)H};
   cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)nb * ld * 4};
-  cuuint32_t box[3] = {32, (cuuint32_t)kDotTile, 1};
+  cuuint32_t box[3] = {32, (cuuint32_t)rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -307,7 +328,7 @@ cudaError_t launch_dot(const SelectArgs& a, int64_t a_terms, int64_t b_terms, in
   CUtensorMap ta, tb, to;
   if (!make_term_map(&ta, a.ws + a_terms, s.nq, s.H, kDotTile) ||
       !make_term_map(&tb, a.ws + b_terms, s.nb, s.H, kDotTile) ||
-      !make_row_map(&to, a.ws + out, s.nq, s.H, s.ld))
+      !make_row_map(&to, a.ws + out, s.nq, s.H, s.ld, 32))
     return cudaErrorInvalidValue;
   DotParams p;
   p.nb = s.nb;
@@ -328,7 +349,7 @@ cudaError_t launch_dot(const SelectArgs& a, int64_t a_terms, int64_t b_terms, in
       cudaFuncSetAttribute(k_dot<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const dim3 grid((ncols + kDotTile - 1) / kDotTile, (s.nqc + kDotTile - 1) / kDotTile, s.H);
-  return launch_pdl(k_dot<MODE>, grid, kDotThreads, smem, st, true, ta, tb, to, p);
+  return launch_pdl(k_dot<MODE>, grid, kDotThreads<MODE>, smem, st, true, ta, tb, to, p);
 }
 
 }  // namespace

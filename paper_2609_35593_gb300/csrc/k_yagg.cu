@@ -36,7 +36,7 @@ namespace ress {
 using namespace ptx;
 
 bool make_term_map(CUtensorMap* m, const void* base, int nb, int H, int rows);
-bool make_row_map(CUtensorMap* m, void* base, int nb, int H, int ld);
+bool make_row_map(CUtensorMap* m, void* base, int nb, int H, int ld, int rows);
 
 namespace {
 
@@ -398,7 +398,7 @@ cudaError_t launch_yagg(const SelectArgs& a, cudaStream_t st) {
   const Shape& s = a.s;
   if (s.ncand <= 0 || s.nqc <= 0) return cudaSuccess;
   CUtensorMap tl, tz;
-  if (!make_row_map(&tl, a.ws + a.L.P, s.nq, s.H, s.ld) ||
+  if (!make_row_map(&tl, a.ws + a.L.P, s.nq, s.H, s.ld, kYRows) ||
       !make_term_map(&tz, a.ws + a.L.zsplit, s.nb, s.H, kYChunk))
     return cudaErrorInvalidValue;
   YParams p;
