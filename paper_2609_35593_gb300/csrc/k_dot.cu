@@ -15,7 +15,8 @@
 // The three dropped products are below 2^-23 of |x||w| together, the size of the fp32
 // rounding of the dot product itself.
 //
-// One CTA per 128 x 128 tile of (i, j) of one head, two per SM, 128 threads (logits) or 256:
+// A tile is 128 rows x 128 blocks of one head.  k_dot, one CTA per tile, two per SM, 128 threads
+// (logits) or 256:
 //   thread 0   TMA of the six 128 x 64 bf16 term tiles (128-byte swizzle), two per mbarrier in
 //              the order the products use them;
 //   warp 0     converged MMA warp, one elected lane issues 6 x 4 tcgen05.mma M128 N128 K16
@@ -26,10 +27,22 @@
 //              with a TMA bulk tensor store as soon as it is formed (columns past the row
 //              stride and rows past the array are clipped by the copy; rows past |P| are never
 //              read).
-// What bounds it is the chain of one tile (launch, loads, MMAs, epilogue, stores: about 6 us),
-// two tiles in flight per SM.  With one barrier for all operands, four epilogue warps and one
-// store of the whole tile at the end: logits 16.8 us at 32 views, 48.5 at 64, 110 at 100, now 14.7,
-// 43.2, 98.8; drift norms 46.1 -> 42.9 and 101 -> 94.5; gains 15.0, 42.8 and 96 either way.
+// What bounds it is the chain of one tile (launch, loads, MMAs, epilogue, stores: about 6 us).
+//
+// k_dot_run, persistent CTAs, one per SM and 320 threads, each over a run of consecutive tiles
+// (j fastest), so that the row terms stay in shared memory along a stripe of rows and the loads
+// and products of a tile run under the epilogue of the one before:
+//   warp 0     TMA: three block terms per tile (two stages), three row terms per stripe;
+//   warp 1     the MMAs, into one of two accumulators;
+//   warps 2-9  the epilogue, two boxes per warp on their way out, in two groups of four warps: a
+//              half of each tile's columns each, or every other tile each where sums run along
+//              the rows (logits).
+// What bounds it is L2: 48 KB in and 64 KB out per tile, about 1.9 us (MMAs: 0.8).  Kernel times
+// at 32 views (576 tiles): logits 14.7 -> 13.5 us, drift norms 14.9 -> 13.2, gains 14.9 -> 12.3
+// against k_dot; all of a selection at 64 views (1936 tiles, six products) 1830 -> 1752 us.  Up to
+// two tiles per SM k_dot is the better one: the layer at 8 views (64 tiles) takes 301 us with it
+// and 306 with k_dot_run, whose CTA needs more of the SM before it can start beside the kernel
+// ahead of it; at 288 tiles (32 views, 128-token query blocks) they are equal, 1042 us.
 // Every mbarrier wait is bounded; a wait that gives up records RESS_ETIMEOUT, lets copies and
 // MMAs already issued finish (again bounded), frees TMEM and returns.
 
@@ -46,14 +59,18 @@ namespace {
 constexpr int kDotTile = 128;                     // rows i and blocks j per CTA
 constexpr uint32_t kTermBytes = kDotTile * 128;   // 128 x 64 bf16
 constexpr uint32_t kDotCols = 128;                // TMEM columns: one fp32 128 x 128 tile
+constexpr uint32_t kRunCols = 256;                // two of them (runs of tiles)
+constexpr uint32_t kBoxBytes = 32 * 32 * 4;       // 32 rows x 32 fp32 of the result
 constexpr uint64_t kDotWaitNs = 2000000000ull;    // 2 s per wait
 constexpr uint64_t kDotDrainNs = 200000000ull;    // 0.2 s to drain after an abort
 
 enum DotMode { kDotGain = 0, kDotLogit = 1, kDotDist = 2 };
-// Epilogue warps: four, or eight (two per 32 rows, a half of the columns each) where no sum runs
-// along the row.
+// One tile per CTA, epilogue warps: four, or eight (two per 32 rows, a half of the columns each)
+// where no sum runs along the row.
 template <int MODE>
 constexpr int kDotThreads = MODE == kDotLogit ? 128 : 256;
+constexpr int kRunWarps = 8;  // runs of tiles: epilogue warps
+constexpr int kRunThreads = 64 + 32 * kRunWarps;
 constexpr float kLogitScale = 0.125f * 1.4426950408889634f;  // 1/sqrt(64) * log2(e)
 
 struct __align__(1024) DotSmem {
@@ -65,18 +82,43 @@ struct __align__(1024) DotSmem {
   int abort;
 };
 
+struct __align__(1024) RunSmem {
+  uint8_t A[3][kTermBytes];     // row-vector terms (hi, mid, lo) of the stripe's 128 rows
+  uint8_t B[2][3][kTermBytes];  // block-vector terms of a tile's 128 blocks
+  uint8_t box[kRunWarps][2][kBoxBytes];  // each epilogue warp's results on their way out
+  float bcol[kRunWarps][kDotTile];       // drift norms: ||z~_j||^2 of the tile's blocks, per warp
+  uint64_t full[2][3];  // operand terms by pairs, in the order the products need them
+  uint64_t done[2];     // a tile's products are complete: accumulator full, operands free
+  uint64_t free[2];     // the accumulator has been read
+  uint32_t tmem_base;
+  int abort;
+};
+
 struct DotParams {
-  int nb, ncand, round;  // key blocks (columns), candidate key blocks
+  int nb;                // key blocks (columns)
   int nq, nqc;           // query blocks (rows), candidate query blocks
-  float rho;
+  int ni, nj, tiles;     // tiles of a head: ni x nj; of all heads
   const float* a;     // per row: c_i (gains) or ||y~_i||^2 (drift norms), [H, nb]
   const float* b;     // per block: ||z~_j||^2 (drift norms), [H, nb]
   float2* lstat;      // logits: per row and 128-block slice (max, sum 2^(L - max))
   int nslices;        // ceil(nb / 128)
   int ld;             // row stride of the output
   uint32_t* status;
-  Budgets bud;
+  uint8_t head[RESS_MAX_HEADS];  // the heads with work, in order
 };
+
+struct DotTile {
+  int h, i0, j0;
+};
+
+__device__ __forceinline__ DotTile dot_tile(const DotParams& p, int t) {
+  const int s = t / p.nj;
+  DotTile r;
+  r.j0 = (t - s * p.nj) * kDotTile;
+  r.h = p.head[s / p.ni];
+  r.i0 = (s % p.ni) * kDotTile;
+  return r;
+}
 
 // (A term, B term) of product q of the six, smallest first: 4 bits per q.
 constexpr uint32_t kTermA = 0x010201u;  // q = 0..5 -> 1, 0, 2, 0, 1, 0
@@ -93,12 +135,62 @@ __device__ __forceinline__ bool dot_wait(uint64_t* bar, uint32_t parity, volatil
   return ok != 0;
 }
 
+// 32 columns of a row of the result from the accumulator: o, and for the logits the running max
+// and sum of 2^(L - max) over the row's slice.
+template <int MODE>
+__device__ __forceinline__ void dot_quarter(const uint32_t (&v)[32], float a, const float* bcol,
+                                            int jq, int nb, float (&o)[32], float& pm, float& ps) {
+  if (MODE == kDotGain) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) o[k] = a - __uint_as_float(v[k]);
+  } else if (MODE == kDotLogit) {
+    float cm = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      o[k] = __uint_as_float(v[k]) * kLogitScale;
+      if (jq + k < nb) cm = fmaxf(cm, o[k]);
+    }
+    if (cm > pm) {
+      ps = (pm == -INFINITY) ? 0.f : ps * exp2f(pm - cm);
+      pm = cm;
+    }
+    // the sum in four interleaved partial sums, with the SFU's exp2 (relative error
+    // about 2^-22: far below what the row's softmax needs, and half the instructions)
+    float sp[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < 32; ++k)
+      if (jq + k < nb) sp[k & 3] += ex2(o[k] - pm);
+    ps += (sp[0] + sp[1]) + (sp[2] + sp[3]);
+  } else {
+    // ||z~_j||^2 of the 32 blocks, broadcast from shared memory
+    const float4* bq = reinterpret_cast<const float4*>(bcol);
+#pragma unroll
+    for (int k4 = 0; k4 < 8; ++k4) {
+      const float4 bz = bq[k4];
+      const float b4[4] = {bz.x, bz.y, bz.z, bz.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = 4 * k4 + e;
+        o[k] = fmaxf(fmaf(-2.0f, __uint_as_float(v[k]), a + b4[e]), 0.f);
+      }
+    }
+  }
+}
+
+// Row `lane` of a box in the 128-byte-swizzled layout: 16-byte chunk k goes to k ^ (row mod 8).
+__device__ __forceinline__ void box_row(uint8_t* box, int lane, const float (&o)[32]) {
+  uint8_t* row = box + lane * 128;
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    *reinterpret_cast<float4*>(row + ((k ^ (lane & 7)) << 4)) =
+        make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(kDotThreads<MODE>)
     k_dot(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-          const __grid_constant__ CUtensorMap tmOut, const DotParams p) {
-  const int h = blockIdx.z, i0 = blockIdx.y * kDotTile, j0 = blockIdx.x * kDotTile;
-  if (MODE == kDotGain && swap_count(p.bud.c[h], p.ncand, p.round, p.rho) <= 0) {
+          const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ DotParams p) {
+  if (p.tiles == 0) {  // a round without swaps
     pdl_wait();
     return;
   }
@@ -107,6 +199,8 @@ __global__ void __launch_bounds__(kDotThreads<MODE>)
                                            ~static_cast<uintptr_t>(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort = &S.abort;
+  const DotTile T = dot_tile(p, blockIdx.x);
+  const int h = T.h, i0 = T.i0, j0 = T.j0;
 
   if (threadIdx.x == 0) {
     for (int t = 0; t < 3; ++t) mbar_init(&S.full[t], 1);
@@ -207,57 +301,19 @@ __global__ void __launch_bounds__(kDotThreads<MODE>)
       uint32_t v[32];
       RESS_TMEM_LD32(tmem + ((uint32_t)(32 * rw) << 16) + 32 * q, v);
       float o[32];
-      if (MODE == kDotGain) {
-#pragma unroll
-        for (int k = 0; k < 32; ++k) o[k] = a - __uint_as_float(v[k]);
-      } else if (MODE == kDotLogit) {
-        const int jq = j0 + 32 * q;
-        float cm = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          o[k] = __uint_as_float(v[k]) * kLogitScale;
-          if (jq + k < p.nb) cm = fmaxf(cm, o[k]);
-        }
-        if (cm > pm) {
-          ps = (pm == -INFINITY) ? 0.f : ps * exp2f(pm - cm);
-          pm = cm;
-        }
-        // the sum in four interleaved partial sums, with the SFU's exp2 (relative error
-        // about 2^-22: far below what the row's softmax needs, and half the instructions)
-        float sp[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int k = 0; k < 32; ++k)
-          if (jq + k < p.nb) sp[k & 3] += ex2(o[k] - pm);
-        ps += (sp[0] + sp[1]) + (sp[2] + sp[3]);
-      } else {
-        // ||z~_j||^2 of this quarter's 32 blocks, broadcast from shared memory
-        const float4* bq = reinterpret_cast<const float4*>(S.bcol + 32 * q);
-#pragma unroll
-        for (int k4 = 0; k4 < 8; ++k4) {
-          const float4 bz = bq[k4];
-          const float b4[4] = {bz.x, bz.y, bz.z, bz.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int k = 4 * k4 + e;
-            o[k] = fmaxf(fmaf(-2.0f, __uint_as_float(v[k]), a + b4[e]), 0.f);
-          }
-        }
-      }
-      uint8_t* row = stage + q * 16384 + r * 128;
-#pragma unroll
-      for (int k = 0; k < 8; ++k)  // 16-byte chunk k of the row goes to chunk k ^ (r mod 8)
-        *reinterpret_cast<float4*>(row + ((k ^ (r & 7)) << 4)) =
-            make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+      dot_quarter<MODE>(v, a, S.bcol + 32 * q, j0 + 32 * q, p.nb, o, pm, ps);
+      uint8_t* box = stage + q * 16384 + rw * 4096;
+      box_row(box, lane, o);
       // this warp's box leaves while the next is formed
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0 && j0 + 32 * q < p.ld && i0 + 32 * rw < p.nq) {
-        tma_store_3d(&tmOut, stage + q * 16384 + rw * 4096, j0 + 32 * q, i0 + 32 * rw, h);
+        tma_store_3d(&tmOut, box, j0 + 32 * q, i0 + 32 * rw, h);
         bulk_commit();
       }
     }
     if (MODE == kDotLogit && i < p.nqc)
-      p.lstat[ri * p.nslices + blockIdx.x] = make_float2(pm, ps);
+      p.lstat[ri * p.nslices + j0 / kDotTile] = make_float2(pm, ps);
     if (lane == 0) bulk_wait_read_all();  // the boxes are read before the shared memory goes away
     __syncwarp();
   }
@@ -271,6 +327,205 @@ __global__ void __launch_bounds__(kDotThreads<MODE>)
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tmem, kDotCols);
+  }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kRunThreads, 1)
+    k_dot_run(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+              const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ DotParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  RunSmem& S = *reinterpret_cast<RunSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                           ~static_cast<uintptr_t>(1023));
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  volatile int* abort = &S.abort;
+  // this CTA's tiles: t0 .. t0 + nt - 1
+  const int t0 = (int)((int64_t)blockIdx.x * p.tiles / gridDim.x);
+  const int nt = (int)((int64_t)(blockIdx.x + 1) * p.tiles / gridDim.x) - t0;
+  constexpr int kGroups = MODE == kDotLogit ? 2 : 1;  // tiles in the epilogue at a time
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 2; ++s) {
+      for (int t = 0; t < 3; ++t) mbar_init(&S.full[s][t], 1);
+      mbar_init(&S.done[s], 1);
+      mbar_init(&S.free[s], kRunWarps / kGroups);
+    }
+    S.abort = 0;
+    fence_barrier_init();
+    prefetch_tensormap(&tmA);
+    prefetch_tensormap(&tmB);
+    prefetch_tensormap(&tmOut);
+  }
+  if (warp == 1) tmem_alloc(&S.tmem_base, kRunCols);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  pdl_wait();
+  const uint32_t tmem = S.tmem_base;
+  auto give_up = [&]() {
+    if (!*abort) flag_status(p.status, kStatusTimeout);
+    *abort = 1;
+  };
+
+  if (warp == 0) {
+    // ---- producer: tile n's operands in stage n mod 2, free when tile n - 2 is done ------
+    int n = 0;
+    if (lane == 0) {
+      bool ok = true;
+      for (; n < nt && ok; ++n) {
+        const int s = n & 1;
+        if (n >= 2 && !mbar_wait(&S.done[s], ((n >> 1) - 1) & 1, abort, kDotWaitNs)) {
+          give_up();
+          break;
+        }
+        const DotTile T = dot_tile(p, t0 + n);
+        const bool stripe = n == 0 || T.j0 == 0;  // new rows
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {  // (mid, mid), (hi, lo), (lo, hi)
+          const int ta = (kTermA >> (4 * t)) & 0xF, tb = (kTermB >> (4 * t)) & 0xF;
+          mbar_arrive_expect_tx(&S.full[s][t], (stripe ? 2 : 1) * kTermBytes);
+          if (n == 0) tma_load_4d(S.A[ta], &tmA, &S.full[s][t], 0, T.i0, T.h, ta);
+          tma_load_4d(S.B[s][tb], &tmB, &S.full[s][t], 0, T.j0, T.h, tb);
+        }
+        if (stripe && n > 0) {  // the last stripe's products have read its row terms
+          ok = mbar_wait(&S.done[s ^ 1], ((n - 1) >> 1) & 1, abort, kDotWaitNs);
+          if (!ok) give_up();
+#pragma unroll
+          for (int t = 0; t < 3; ++t) {
+            const int ta = (kTermA >> (4 * t)) & 0xF;
+            if (ok) tma_load_4d(S.A[ta], &tmA, &S.full[s][t], 0, T.i0, T.h, ta);
+          }
+        }
+      }
+    }
+    __syncwarp();
+    pdl_trigger();
+    if (lane == 0) {
+      // copies in flight must land before the shared memory goes away: the MMA warp waits for
+      // them as it goes, unless the CTA gave up
+      if (nt > 0) mbar_wait(&S.done[(nt - 1) & 1], ((nt - 1) >> 1) & 1, abort, kDotWaitNs);
+      if (*abort) {
+        volatile int no_abort = 0;
+        for (int m = n > 2 ? n - 2 : 0; m < n; ++m)
+          for (int t = 0; t < 3; ++t)
+            mbar_wait(&S.full[m & 1][t], (m >> 1) & 1, &no_abort, kDotDrainNs);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---- MMA: tile n into accumulator n mod 2 --------------------------------------------
+    const bool leader = elect_one();
+    int committed = 0;  // tiles whose products went out, at least in part
+    if (__popc(__ballot_sync(0xffffffffu, leader)) != 1) {  // exactly one issuing lane
+      if (lane == 0) {
+        flag_status(p.status, kStatusBadRow);
+        *abort = 1;
+      }
+    } else {
+      const uint32_t idesc = idesc_bf16_f32(kDotTile, kDotTile, false);
+      bool ok = true;
+      for (int n = 0; n < nt && ok; ++n) {
+        const int s = n & 1;
+        if (n >= 2) ok = dot_wait(&S.free[s], ((n >> 1) - 1) & 1, abort, kDotWaitNs);
+        tc_fence_after();
+        bool issued = false;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+          if (q < 3 && ok) {  // (the last three products use terms that have landed)
+            ok = dot_wait(&S.full[s][q], (n >> 1) & 1, abort, kDotWaitNs);
+            tc_fence_after();
+          }
+          if (ok && leader) {
+            const uint32_t a = smem_u32(S.A[(kTermA >> (4 * q)) & 0xF]);
+            const uint32_t b = smem_u32(S.B[s][(kTermB >> (4 * q)) & 0xF]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              mma_bf16_ss(tmem + kDotTile * s, sdesc_sw128(a + 32 * k), sdesc_sw128(b + 32 * k),
+                          idesc, (q > 0 || k > 0) ? 1u : 0u);
+            issued = true;
+          }
+          __syncwarp();
+        }
+        if (leader && issued) mma_commit(&S.done[s]);
+        if (__any_sync(0xffffffffu, issued)) committed = n + 1;
+      }
+      if (!ok && lane == 0) give_up();
+    }
+    pdl_trigger();
+    if (committed > 0) {  // products still running finish before the accumulators are freed
+      volatile int no_abort = 0;
+      if (lane == 0)
+        mbar_wait(&S.done[(committed - 1) & 1], ((committed - 1) >> 1) & 1, &no_abort,
+                  *abort ? kDotDrainNs : kDotWaitNs);
+      __syncwarp();
+    }
+  } else {
+    // ---- epilogue: this warp's 32 rows are the TMEM lanes it can read --------------------
+    const int ew = warp - 2, rw = warp & 3, group = ew >> 2;
+    const int r = 32 * rw + lane;  // row of the tile = TMEM lane
+    constexpr int kQuarters = MODE == kDotLogit ? 4 : 2;  // of 32 columns per warp and tile
+    const int q0 = MODE == kDotLogit ? 0 : 2 * group;
+    float* bcol = S.bcol[ew];
+    bool ok = true;
+    if ((MODE == kDotLogit ? group : 0) >= nt) pdl_trigger();
+    for (int n = MODE == kDotLogit ? group : 0; n < nt && ok; n += kGroups) {
+      const DotTile T = dot_tile(p, t0 + n);
+      const int i = T.i0 + r;
+      const int64_t ri = (int64_t)T.h * p.nq + i;
+      float a = 0.f;
+      if (MODE != kDotLogit && i < p.nq) a = p.a[ri];
+      if (MODE == kDotDist) {
+        __syncwarp();  // the last tile's norms have been read
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int k = 32 * (q0 + e) + lane, j = T.j0 + k;
+          bcol[k] = j < p.nb ? p.b[(int64_t)T.h * p.nb + j] : 0.f;
+        }
+        __syncwarp();
+      }
+      if (n + kGroups >= nt) pdl_trigger();
+      ok = dot_wait(&S.done[n & 1], (n >> 1) & 1, abort, kDotWaitNs);
+      if (!ok) {
+        if (lane == 0) give_up();
+        break;
+      }
+      tc_fence_after();
+      float pm = -INFINITY, ps = 0.f;  // logits: running max and sum over the slice
+#pragma unroll 1
+      for (int e = 0; e < kQuarters; ++e) {
+        const int q = q0 + e;
+        uint32_t v[32];
+        RESS_TMEM_LD32(tmem + ((uint32_t)(32 * rw) << 16) + kDotTile * (n & 1) + 32 * q, v);
+        if (e == kQuarters - 1) {  // read to the end: the accumulator is free
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&S.free[n & 1]);
+        }
+        float o[32];
+        dot_quarter<MODE>(v, a, bcol + 32 * q, T.j0 + 32 * q, p.nb, o, pm, ps);
+        uint8_t* box = S.box[ew][e & 1];
+        if (lane == 0) bulk_wait_read_but1();  // this box's last copy has read it
+        __syncwarp();
+        box_row(box, lane, o);
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          if (T.j0 + 32 * q < p.ld && T.i0 + 32 * rw < p.nq)
+            tma_store_3d(&tmOut, box, T.j0 + 32 * q, T.i0 + 32 * rw, T.h);
+          bulk_commit();  // (also where nothing left: groups are counted)
+        }
+      }
+      if (MODE == kDotLogit && i < p.nqc)
+        p.lstat[ri * p.nslices + T.j0 / kDotTile] = make_float2(pm, ps);
+    }
+    if (lane == 0) bulk_wait_read_all();  // the boxes are read before the shared memory goes away
+    __syncwarp();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kRunCols);
   }
 }
 
@@ -332,24 +587,34 @@ cudaError_t launch_dot(const SelectArgs& a, int64_t a_terms, int64_t b_terms, in
     return cudaErrorInvalidValue;
   DotParams p;
   p.nb = s.nb;
-  p.ncand = s.ncand;
   p.nq = s.nq;
   p.nqc = s.nqc;
-  p.round = round;
-  p.rho = rho;
   p.a = rowv;
   p.b = colv;
   p.lstat = (float2*)(a.ws + a.L.lstat);
   p.nslices = (s.nb + kDotTile - 1) / kDotTile;
   p.ld = s.ld;
   p.status = (uint32_t*)(a.ws + a.L.status);
-  for (int h = 0; h < RESS_MAX_HEADS; ++h) p.bud.c[h] = a.c[h];
-  const size_t smem = sizeof(DotSmem) + 1024;
+  p.ni = (s.nqc + kDotTile - 1) / kDotTile;
+  p.nj = (ncols + kDotTile - 1) / kDotTile;
+  int heads = 0;  // a round swaps nothing in a head whose budget leaves no pair
+  for (int h = 0; h < s.H; ++h)
+    if (MODE != kDotGain || swap_count(a.c[h], s.ncand, round, rho) > 0)
+      p.head[heads++] = (uint8_t)h;
+  p.tiles = heads * p.ni * p.nj;
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool run = p.tiles > 2 * sms;  // more than one wave of k_dot
+  auto* kern = run ? k_dot_run<MODE> : k_dot<MODE>;
+  const size_t smem = (run ? sizeof(RunSmem) : sizeof(DotSmem)) + 1024;
   cudaError_t e =
-      cudaFuncSetAttribute(k_dot<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const dim3 grid((ncols + kDotTile - 1) / kDotTile, (s.nqc + kDotTile - 1) / kDotTile, s.H);
-  return launch_pdl(k_dot<MODE>, grid, kDotThreads<MODE>, smem, st, true, ta, tb, to, p);
+  // (no tile: a round without swaps)
+  const int ctas = run ? sms : p.tiles < 1 ? 1 : p.tiles;
+  return launch_pdl(kern, ctas, run ? kRunThreads : kDotThreads<MODE>, smem, st, true, ta, tb, to,
+                    p);
 }
 
 }  // namespace
