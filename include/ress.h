@@ -233,8 +233,9 @@ int ress_sparse_attn_f32(const ress_dims* dims, const uint16_t* Q, const uint16_
  * attention starts without the union pass of ress_sparse_attn.  The CSR and J_best are bit
  * for bit those of the three separate calls.  O is too on the 128-token query grid; on the
  * 64-token grid the forward pairs the candidate query blocks by the overlap of their kept
- * lists (ress_sparse_attn pairs adjacent blocks), which changes only the order in which a
- * row takes its own kept blocks, so O agrees with the separate calls' to rounding (and is
+ * lists (ress_sparse_attn pairs adjacent blocks), and where the items of a layer leave SMs
+ * idle up to four CTAs share an item's blocks; both change only the order in which a row takes
+ * its own kept blocks, so O agrees with the separate calls' to rounding (and is
  * deterministic). */
 int ress_forward(const ress_dims* dims, const uint16_t* Q, const uint16_t* K, const uint16_t* V,
                  const float* F, const int32_t* c_h_host, int32_t rounds, float rho, void* ws,
