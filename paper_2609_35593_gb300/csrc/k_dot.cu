@@ -37,7 +37,8 @@
 //   warps 2-9  the epilogue, two boxes per warp on their way out, in two groups of four warps: a
 //              half of each tile's columns each, or every other tile each where sums run along
 //              the rows (logits).
-// What bounds it is L2: 48 KB in and 64 KB out per tile, about 1.9 us (MMAs: 0.8).  Kernel times
+// What bounds it is L2: 48 KB in and 64 KB out per tile, about 1.9 us (at 64 views a copy that
+// stores every box twice takes 42 us instead of 28, one with a sixth of the MMAs 27).  Kernel times
 // at 32 views (576 tiles): logits 14.7 -> 13.5 us, drift norms 14.9 -> 13.2, gains 14.9 -> 12.3
 // against k_dot; at 100 views (4624 tiles) 98.8 -> 67.9, 94.5 -> 67.9 and 96 -> 64.6; all of a
 // selection at 64 views (1936 tiles, six products) 1830 -> 1752 us.  Up to
