@@ -6,11 +6,12 @@
 // k_dot left in lstat.  P overwrites L in place; y~ is written in fp32, as three bf16
 // terms (the row operand of the drift-norm products) and as ||y~_i||^2.
 //
-// One CTA per 128 candidate rows of a head and part of the key blocks (the blocks are split
-// into `parts` consecutive ranges of chunks when that fills more of the GPU; each part's
-// partial y~ goes to scratch and the CTA that finishes last sums the parts in their order and
-// writes the outputs, so the result does not depend on which finishes first), 544 threads,
-// 64 key blocks per chunk, two pipeline stages:
+// Where the stripes of 128 candidate rows leave SMs idle, the key blocks are summed as up to three
+// consecutive ranges of chunks, added up in their order.  Long ranges (launch_yagg draws the line)
+// go to a CTA each: each range's partial y~ goes to scratch and the CTA that finishes last adds
+// them and writes the outputs, so the result does not depend on which finishes first.  Short ones
+// stay in one CTA with a TMEM accumulator each: the same sums to the bit.  544 threads, 64 key
+// blocks per chunk, two pipeline stages:
 //   warp 16    lane 0 loads chunk c + 1 by TMA (L: two 32-column fp32 boxes; z~: its three
 //              bf16 term tiles, 64 blocks x 64 channels) while the chunk c is converted;
 //              then the converged warp, one elected lane, issues the chunk's MMAs
@@ -46,7 +47,8 @@ constexpr int kMmaWarp = kConvWarps;
 constexpr int kYRows = 128;      // candidate rows per CTA
 constexpr int kYChunk = 64;      // key blocks per pipeline step
 constexpr int kYStages = 2;
-constexpr uint32_t kYCols = 64;  // TMEM columns: y~ (128 x 64 fp32)
+constexpr uint32_t kYCols = 64;  // TMEM columns: y~ (128 x 64 fp32) of one range
+constexpr int kYMaxRanges = 3;
 constexpr uint64_t kYWaitNs = 2000000000ull;
 constexpr uint64_t kYDrainNs = 200000000ull;
 
@@ -72,7 +74,8 @@ struct YParams {
   float* ny;        // [H, nb]
   int64_t term_words;  // H nb 32
   uint32_t* status;
-  int parts;           // key-block parts per stripe of 128 rows
+  int parts;           // CTAs per stripe, a range of chunks each
+  int ranges;          // ranges of a CTA: one if parts > 1
   float* part_buf;     // [parts][H][nq][64] partial y~ (parts > 1)
   uint32_t* arrivals;  // [H][stripes] parts done, zero before the launch (parts > 1)
 };
@@ -126,7 +129,8 @@ __global__ void __launch_bounds__(kYThreads, 1)
     prefetch_tensormap(&tmL);
     prefetch_tensormap(&tmZ);
   }
-  if (warp == kMmaWarp) tmem_alloc(&S.tmem_base, kYCols);
+  const uint32_t ncols = p.ranges > 1 ? 4 * kYCols : kYCols;  // (a power of two)
+  if (warp == kMmaWarp) tmem_alloc(&S.tmem_base, ncols);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -160,7 +164,12 @@ __global__ void __launch_bounds__(kYThreads, 1)
     };
     const uint32_t idesc = idesc_bf16_f32(kYRows, 64, true);
     if (!failed && !produce(0)) failed = true;
+    int range = 0, rbegin = 0;  // this chunk's range and its first chunk
     for (int c = 0; c < nch && !failed; ++c) {
+      if (c == nch * (range + 1) / p.ranges) {
+        ++range;
+        rbegin = c;
+      }
       if (c + 1 < nch && !produce(c + 1)) {
         failed = true;
         break;
@@ -178,8 +187,8 @@ __global__ void __launch_bounds__(kYThreads, 1)
           const uint32_t b = smem_u32(S.Z[s][(kTermB >> (4 * q)) & 0xF]);
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            mma_bf16_ss(tmem, sdesc_sw128(a + 32 * k), sdesc_sw128(b + 2048 * k), idesc,
-                        (c > 0 || q > 0 || k > 0) ? 1u : 0u);
+            mma_bf16_ss(tmem + kYCols * range, sdesc_sw128(a + 32 * k), sdesc_sw128(b + 2048 * k),
+                        idesc, (c > rbegin || q > 0 || k > 0) ? 1u : 0u);
         }
         mma_commit(&S.empty[s]);
         if (c + 1 == nch) mma_commit(&S.done);
@@ -286,7 +295,15 @@ __global__ void __launch_bounds__(kYThreads, 1)
     uint32_t v[16];
     if (!failed && y_wait(&S.done, 0, abort)) {
       tc_fence_after();
-      RESS_TMEM_LD16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * qq, v);
+      const uint32_t acc = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * qq;
+      RESS_TMEM_LD16(acc, v);
+      for (int t = 1; t < p.ranges; ++t) {
+        uint32_t w[16];
+        RESS_TMEM_LD16(acc + kYCols * t, w);
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          v[k] = __float_as_uint(__uint_as_float(v[k]) + __uint_as_float(w[k]));
+      }
       have = true;
     } else if (lane == 0) {
       y_give_up(S, p.status);
@@ -368,22 +385,33 @@ __global__ void __launch_bounds__(kYThreads, 1)
   }
   if (warp == kMmaWarp) {
     tc_fence_after();
-    tmem_dealloc(tmem, kYCols);
+    tmem_dealloc(tmem, ncols);
   }
 }
 
 // One CTA per SM: when the stripes of rows leave SMs idle, split the key blocks into as many
-// parts (up to 3) as still run in one wave.  (A second wave costs more than the split saves:
-// measured at 32 views on 64-token query blocks, 96 stripes.)  The partial sums of k parts
+// ranges (up to 3) as still run in one wave.  (A second wave costs more than the split saves:
+// measured at 32 views on 64-token query blocks, 96 stripes.)  The partial sums of k ranges
 // take 64 k of the ld floats per row of the gains array.
-int yagg_parts(const Shape& s) {
+int yagg_ranges(const Shape& s) {
   const int stripes = (s.nqc + kYRows - 1) / kYRows, nchunks = (s.nb + kYChunk - 1) / kYChunk;
-  int dev = 0, sms = 1, parts = 1;
+  int dev = 0, sms = 1, ranges = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  for (int k = 2; k <= 3 && k <= nchunks && 64 * k <= s.ld; ++k)
-    if ((int64_t)stripes * s.H * k <= sms) parts = k;
-  return parts;
+  for (int k = 2; k <= kYMaxRanges && k <= nchunks && 64 * k <= s.ld; ++k)
+    if ((int64_t)stripes * s.H * k <= sms) ranges = k;
+  return ranges;
+}
+
+// A CTA per range where that takes at least 6 chunks off a CTA's chain of them: handing partial
+// sums over through scratch (stores, fence, counter, loads) costs about as much as 6 chunks.
+// Layer with a CTA per range against all ranges in one CTA, three ranges, 16 heads: 3 chunks
+// (8 views) 222.5 and 214.4 us, 5 (12 views) 318.2 and 311.9, 6 (16) 448.6 and 445.7, 128-token
+// query blocks 6 (16) 378.8 and 372.5, 9 (24) 684.0 and 684.5, 11 (32) 1036.4 and 1039.4.  The
+// 8-view kernel itself takes 14.1 us instead of 20.0.
+int yagg_parts(const Shape& s) {
+  const int nchunks = (s.nb + kYChunk - 1) / kYChunk, k = yagg_ranges(s);
+  return nchunks - (nchunks + k - 1) / k >= 6 ? k : 1;
 }
 
 }  // namespace
@@ -417,6 +445,7 @@ cudaError_t launch_yagg(const SelectArgs& a, cudaStream_t st) {
   p.status = (uint32_t*)(a.ws + a.L.status);
   const int stripes = (s.nqc + kYRows - 1) / kYRows;
   p.parts = yagg_parts(s);
+  p.ranges = p.parts > 1 ? 1 : yagg_ranges(s);
   // scratch while the selection scores: the gains array (partial y~) and the attention
   // items' length array (arrival counts), both unused until the restoration rounds
   p.part_buf = (float*)(a.ws + a.L.t);
