@@ -30,8 +30,6 @@
 // issued finish (again bounded); the pair then meets at a cluster barrier, frees TMEM and
 // returns.
 
-#include <climits>
-
 #include <cudaTypedefs.h>
 
 #include "ress_internal.cuh"
@@ -111,6 +109,18 @@ __device__ __forceinline__ bool o_epi_sync_and(int hf, bool v) {
       : "memory");
   return r != 0;
 }
+// The same of all eight epilogue warps (drift).
+__device__ __forceinline__ bool o_epi_sync_and_all(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 5, 256, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(v ? 1u : 0u)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void o_epi_sync_all() { asm volatile("bar.sync 5, 256;" ::: "memory"); }
 __device__ __forceinline__ void o_epi_sync(int hf) {
   asm volatile("bar.sync %0, 128;" ::"r"(3 + hf) : "memory");
 }
@@ -119,15 +129,20 @@ __device__ __forceinline__ void o_epi_sync(int hf) {
 struct OUnit {
   int mt, col, width;
 };
-// Drift: a cluster of p.group pairs per stripe, which take its channel tiles in turn.
+// Drift: persistent pairs over whole stripes, or a cluster of p.group pairs per stripe, which take
+// its channel tiles in turn.
 template <int MODE>
 __device__ __forceinline__ int units_of_pair(const OParams& p) {
+  if (MODE == kDrift && p.group == 1)
+    return ((p.mtiles - 1 - (int)(blockIdx.x >> 1)) / (int)(gridDim.x >> 1) + 1) * p.ntiles;
   if (MODE == kDrift) return (p.ntiles - 1 - (int)(cluster_rank() >> 1)) / p.group + 1;
   const int units = p.whole + (p.mtiles * p.ntiles - p.whole) * p.parts;
   return (units - 1 - (int)(blockIdx.x >> 1)) / (int)(gridDim.x >> 1) + 1;
 }
 template <int MODE>
 __device__ __forceinline__ OUnit unit_of_pair(const OParams& p, int k) {
+  if (MODE == kDrift && p.group == 1)
+    return OUnit{(int)(blockIdx.x >> 1) + k / p.ntiles * (int)(gridDim.x >> 1), kON * (k % p.ntiles), kON};
   if (MODE == kDrift)
     return OUnit{(int)blockIdx.x / (2 * p.group), kON * ((int)(cluster_rank() >> 1) + k * p.group), kON};
   // consecutive tiles share their token stripe, so O slices are re-read from L2
@@ -326,7 +341,7 @@ __global__ void __launch_bounds__(kOThreads, 1)
       }
       bool ok = o_wait(&C.acc_full[b], use & 1, abort);
       if (MODE == kResidual && p.has_x && ok && boxes > 0) ok = o_wait(&C.x_full[hf], k & 1, abort);
-      if (!o_epi_sync_and(hf, ok)) {  // the four warps leave together
+      if (!(MODE == kDrift ? o_epi_sync_and_all(ok) : o_epi_sync_and(hf, ok))) {  // all leave together
         if (!ok && lane == 0) o_give_up(C, p.status);
         break;
       }
@@ -368,6 +383,25 @@ __global__ void __launch_bounds__(kOThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(cluster_addr(&C.acc_empty[b], lead));  // may be reused
+      if (MODE == kDrift && p.group == 1 && (k + 1) % p.ntiles == 0) {
+        // the stripe is complete: rows over their channel halves, 64-token blocks over their rows,
+        // warp tree by warp tree (as after a cluster's tiles, below)
+        C.rowsum[hf][r] = rowsum;
+        rowsum = 0.f;
+        o_epi_sync_all();
+        if (hf == 0) {
+          float v = 0.f;
+#pragma unroll
+          for (int q = 0; q < 2; ++q) v += C.rowsum[q][r];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane == 0) C.blocksum[quarter] = v;
+        }
+        o_epi_sync_all();
+        const int blk = 2 * (2 * t.mt + rank) + (quarter >> 1);
+        if (hf == 0 && lane == 0 && (quarter & 1) == 0 && blk < p.nb && !*abort)
+          p.drift[blk] = C.blocksum[quarter] + C.blocksum[quarter + 1];
+      }
       if (MODE == kResidual) {
         fence_proxy_async_smem();
         o_epi_sync(hf);
@@ -382,13 +416,13 @@ __global__ void __launch_bounds__(kOThreads, 1)
         }
       }
     }
-    if (MODE == kDrift) C.rowsum[hf][r] = rowsum;
+    if (MODE == kDrift && p.group > 1) C.rowsum[hf][r] = rowsum;
     if (leader) bulk_wait_read_all();
   }
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // the pair's MMAs and barrier arrivals are over in both CTAs
-  if (MODE == kDrift) {
+  if (MODE == kDrift && p.group > 1) {
     // the cluster's first pair sums its rows over the pairs (and their channel halves) in
     // order, then each 64-token block over its rows, warp tree by warp tree
     if (cluster_rank() < 2 && threadIdx.x < kOM) {
@@ -473,23 +507,29 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
     p.parts = 4 * left <= slots ? 4 : 2;
   }
   const int units = p.whole + (tiles - p.whole) * p.parts;
-  // Drift: as many pairs per stripe (a cluster) as make the fewest tiles in a row per SM; a
-  // GPC rarely has room for as many clusters of 8 CTAs as its SMs would allow, so those are
-  // counted with one in eight less (8 views: 43 stripes of 4 tiles leave 66 of 152 SMs idle
-  // with one pair each: 45.3 us, 41.2 with four; 16 views 89.8 and, with two, 73.1).
+  // Drift: one pair per stripe, persistent over the stripes, or a cluster of 2 or 4 pairs.  The
+  // cost of a tile is its K / 64 steps and an epilogue of about two; starting and ending a CTA is
+  // about eight, once for persistent pairs and for every wave of clusters.  A GPC rarely has room
+  // for as many clusters of 8 CTAs as its SMs would allow, so those are counted with one in eight
+  // less.  (8 views, 16 heads: 47.6 us with a pair per stripe, 50.4 in clusters of two, 44.3 of
+  // four; 16 views 94.7, 75.3 and 87.4.  84,608 tokens, 8 heads: 71.3 us with persistent pairs, 83.9
+  // with a CTA pair launched per stripe, 98.0 in clusters of two; 4 heads 25.6 and 39.2.)
   p.group = 1;
   if (MODE == kDrift) {
-    int best = INT_MAX;
+    int64_t best = INT64_MAX;
     for (int g = 1; g <= 4 && g <= p.ntiles; g *= 2) {
       const int fit = max(1, g == 4 ? slots * 7 / 32 : slots / g);
-      const int rounds = (p.mtiles + fit - 1) / fit * ((p.ntiles + g - 1) / g);
-      if (rounds < best) {
-        best = rounds;
+      const int64_t waves = (p.mtiles + fit - 1) / fit, tile = p.K / 64 + 2;
+      const int64_t run = (p.ntiles + g - 1) / g * tile;
+      const int64_t cost = g == 1 ? waves * run + 8 : waves * (run + 8);
+      if (cost < best) {
+        best = cost;
         p.group = g;
       }
     }
   }
-  const int ctas = 2 * (MODE == kDrift ? p.mtiles * p.group : min(units, slots));
+  const int ctas =
+      2 * (p.group > 1 ? p.mtiles * p.group : min(MODE == kDrift ? p.mtiles : units, slots));
   tbp = tb;
   if (p.parts > 1 && !make_bf16_map(&tbp, a.W_o, a.Dm, K, kON / 2 / p.parts))
     return cudaErrorInvalidValue;

@@ -15,6 +15,8 @@ pytestmark = pytest.mark.gpu
     (9700, 2, 512),     # 76 tiles: one whole wave of 76 pairs
     (9985, 2, 512),     # two tiles more than a wave
     (14000, 1, 768),    # 165 tiles: 13 past two waves
+    (256 * 77 + 1, 2, 256),   # drift: pairs with one stripe and with two
+    (256 * 160 - 70, 1, 320), # two and three stripes of two channel tiles
 ])
 def test_pair_tile_edges(N, H, d_model):
     import paper_2609_35593_gb300 as ress
