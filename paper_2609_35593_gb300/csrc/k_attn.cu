@@ -163,13 +163,10 @@ __device__ __forceinline__ void give_up(AttnSmem& S, uint32_t* status) {
 // 128-token query blocks (one block per 128-row item) the list is the block's own, every
 // entry kept by both halves.  One warp per item; grid ceil(H * npairs / 8) x 256 threads.
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_pairs(const int32_t* __restrict__ row_ptr,
-                                               const int32_t* __restrict__ col_idx,
-                                               int64_t cap, int64_t scratch_cap, int nb,
-                                               int npairs, int H, bool qb128,
-                                               int32_t* __restrict__ plist,
-                                               int32_t* __restrict__ plen, uint32_t* status,
-                                               uint32_t* counter) {
+__global__ void __launch_bounds__(256)
+    k_pairs(const int32_t* row_ptr, const int32_t* col_idx, int64_t cap, int64_t scratch_cap, int nb,
+            int npairs, int H, bool qb128, int32_t* plist, int32_t* plen, uint32_t* status,
+            uint32_t* counter) {
   __shared__ uint32_t bits[8][2][RESS_MAX_BLOCKS / 32];
   pdl_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

@@ -104,16 +104,10 @@ __device__ __forceinline__ float warp_sum(float v) {
 // key blocks), each over the valid tokens of its block.  grid (nb, 3); one token is H*64
 // bf16 = 8H 16-byte chunks (H <= 32).
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_pool(const uint16_t* __restrict__ Q,
-                                                    const uint16_t* __restrict__ K,
-                                                    const uint16_t* __restrict__ V, int N,
-                                                    int H, int nb, int qb, int nq,
-                                                    float* __restrict__ qbar,
-                                                    float* __restrict__ kbar,
-                                                    float* __restrict__ vbar,
-                                                    uint16_t* __restrict__ qsplit,
-                                                    uint16_t* __restrict__ ksplit,
-                                                    uint32_t* __restrict__ zero, int nzero) {
+__global__ void __launch_bounds__(kThreads)
+    k_pool(const uint16_t* Q, const uint16_t* K, const uint16_t* V, int N, int H, int nb, int qb,
+           int nq, float* qbar, float* kbar, float* vbar, uint16_t* qsplit, uint16_t* ksplit,
+           uint32_t* zero, int nzero) {
   __shared__ float part[kThreads * 8];
   const int j = blockIdx.x, which = blockIdx.y;
   ptx::pdl_wait();
@@ -171,12 +165,9 @@ __global__ void __launch_bounds__(kThreads) k_pool(const uint16_t* __restrict__ 
 // F_h and the 16 pooled values sit in shared memory with rows padded to 68 floats, so that
 // the float4 reads of a warp (32 channels, one column group) hit every bank once per pass.
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kThreads) k_zproj(const float* __restrict__ F,
-                                                     const float* __restrict__ vbar, int nb,
-                                                     float* __restrict__ ztil,
-                                                     uint16_t* __restrict__ zsplit,
-                                                     int64_t term_stride,
-                                                     float* __restrict__ nz) {
+__global__ void __launch_bounds__(kThreads)
+    k_zproj(const float* F, const float* vbar, int nb, float* ztil, uint16_t* zsplit,
+            int64_t term_stride, float* nz) {
   constexpr int kPad = 68;
   __shared__ __align__(16) float Fs[64][kPad];  // Fs[a][b] = F[a][b]
   __shared__ __align__(16) float Vs[16][kPad];
@@ -1336,9 +1327,9 @@ __global__ void __launch_bounds__(32 * kRowWarps, LARGE ? 8 : 10) k_round_rows(S
 // result by rounding alone.  grid (windows, H) x 512 threads: all warps form the
 // window's overlaps, then take the pairs by weight (one block-wide maximum per pair).
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(512) k_pairing(const uint32_t* __restrict__ bmask, int nq,
-                                                 int words, int ncand, int npaired, int items,
-                                                 int32_t* __restrict__ prow) {
+__global__ void __launch_bounds__(512)
+    k_pairing(const uint32_t* bmask, int nq, int words, int ncand, int npaired, int items,
+              int32_t* prow) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ptx::pdl_wait();
   constexpr int W = kPairWindow;
@@ -1475,9 +1466,8 @@ struct CsrOut {
 // Row offsets of variable-length kept lists (CDF threshold): row_ptr = exclusive scan of the
 // kept counts over the H * nq rows (candidate rows: kcount; special query rows: nb).  One
 // CTA of 1024 threads, each owning a contiguous run of rows.
-__global__ void __launch_bounds__(1024) k_rowptr(const int32_t* __restrict__ kcount, int H,
-                                                 int nq, int nqc, int nb,
-                                                 int32_t* __restrict__ row_ptr) {
+__global__ void __launch_bounds__(1024)
+    k_rowptr(const int32_t* kcount, int H, int nq, int nqc, int nb, int32_t* row_ptr) {
   __shared__ long long wsum[32];
   ptx::pdl_wait();
   const long long R = (long long)H * nq;

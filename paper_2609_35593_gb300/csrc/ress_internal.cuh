@@ -139,12 +139,14 @@ __device__ __forceinline__ void split3_bf16x2(float x0, float x1, uint32_t& hi, 
   lo = cvt_bf16x2(s0, s1);
 }
 
-// Streaming 16-byte load that bypasses L1 allocation (read-once inputs).
+// Streaming 16-byte load that bypasses L1 allocation (read-once inputs).  Coherent: the inputs may
+// be the output of a kernel that this one overlaps (ptx::pdl_wait), which rules out ld.global.nc.
 __device__ __forceinline__ uint4 ld_stream(const uint4* p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w)
-               : "l"(p));
+               : "l"(p)
+               : "memory");
   return r;
 }
 

@@ -24,7 +24,10 @@ __device__ __forceinline__ bool elect_one() {
 
 // Programmatic dependent launch (kernels started by launch_pdl, ress_internal.cuh).  wait: until
 // every earlier kernel of the stream has completed and its writes are visible; every kernel
-// waits, in every CTA, before its first access to global memory.  trigger: the next kernel of
+// waits, in every CTA, before its first access to global memory.  Data that the kernel ahead
+// writes changes while this one is running, so no pointer parameter of such a kernel is
+// __restrict__ and nothing is read with ld.global.nc (which is for data that is constant for the
+// whole kernel, and which the compiler may hoist over the wait).  trigger: the next kernel of
 // the stream may start its CTAs once every CTA of this one has triggered or ended.  It stands
 // after the wait and late in each kernel, when the CTA has only its last stage left: a trigger
 // at the top lets several later kernels queue up on the SMs, whose CTAs then sit unevenly
