@@ -628,6 +628,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
                   m_use = mt;
                   rescale = true;
                 }
+                __syncwarp();
                 exps(x, m_use, w);
               }
             }

@@ -301,6 +301,7 @@ __global__ void __launch_bounds__(kDotThreads<MODE>)
 #pragma unroll 1
     for (int q = q0; q < q0 + kQuarters; ++q) {
       uint32_t v[32];
+      __syncwarp();  // lane 0 comes from the store below
       RESS_TMEM_LD32(tmem + ((uint32_t)(32 * rw) << 16) + 32 * q, v);
       float o[32];
       dot_quarter<MODE>(v, a, S.bcol + 32 * q, j0 + 32 * q, p.nb, o, pm, ps);
@@ -497,6 +498,7 @@ __global__ void __launch_bounds__(kRunThreads, 1)
       for (int e = 0; e < kQuarters; ++e) {
         const int q = q0 + e;
         uint32_t v[32];
+        __syncwarp();  // lane 0 comes from the store below
         RESS_TMEM_LD32(tmem + ((uint32_t)(32 * rw) << 16) + kDotTile * (n & 1) + 32 * q, v);
         if (e == kQuarters - 1) {  // read to the end: the accumulator is free
           tc_fence_before();

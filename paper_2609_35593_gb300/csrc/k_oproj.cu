@@ -100,6 +100,7 @@ __device__ __forceinline__ void o_give_up(OCtl& C, uint32_t* status) {
 // Named barriers of the four epilogue warps of channel half hf (0 or 1); the first also ANDs
 // a flag across them.
 __device__ __forceinline__ bool o_epi_sync_and(int hf, bool v) {
+  __syncwarp();
   uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
@@ -111,6 +112,7 @@ __device__ __forceinline__ bool o_epi_sync_and(int hf, bool v) {
 }
 // The same of all eight epilogue warps (drift).
 __device__ __forceinline__ bool o_epi_sync_and_all(bool v) {
+  __syncwarp();
   uint32_t r;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
@@ -120,8 +122,12 @@ __device__ __forceinline__ bool o_epi_sync_and_all(bool v) {
       : "memory");
   return r != 0;
 }
-__device__ __forceinline__ void o_epi_sync_all() { asm volatile("bar.sync 5, 256;" ::: "memory"); }
+__device__ __forceinline__ void o_epi_sync_all() {
+  __syncwarp();
+  asm volatile("bar.sync 5, 256;" ::: "memory");
+}
 __device__ __forceinline__ void o_epi_sync(int hf) {
+  __syncwarp();
   asm volatile("bar.sync %0, 128;" ::"r"(3 + hf) : "memory");
 }
 

@@ -95,6 +95,7 @@ __device__ __forceinline__ bool y_wait(uint64_t* bar, uint32_t parity, volatile 
 
 // Barrier among the converter warps only (named barrier 1; the MMA warp takes no part).
 __device__ __forceinline__ void conv_sync() {
+  __syncwarp();
   asm volatile("bar.sync 1, %0;" ::"n"(32 * kConvWarps) : "memory");
 }
 

@@ -61,3 +61,41 @@ def test_overlapped_kernels_promise_nothing_about_aliasing(name, params):
 def test_no_read_only_loads():
     for path in glob.glob(os.path.join(CSRC, "*.cu*")):
         assert not re.search(r"ld\.global\.nc|__ldg\b|\.nc\.", _code(path)), path
+
+
+def _helpers():
+    """(file:name, body) of every device function with an instruction that is .aligned over the
+    warp besides TMEM loads and stores (bar.* without .cta is short for barrier.cta.aligned)."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        text = _code(path)
+        for m in re.finditer(r"__device__ __forceinline__ [\w ]+?\b(\w+)\(", text):
+            params = _balanced(text, m.end() - 1, "()")
+            body = _balanced(text, text.index("{", m.end() - 1 + len(params)), "{}")
+            if re.search(r'barrier\.cluster|"bar\.|tcgen05\.(?:de)?alloc', body):
+                out.append((m.group(1), body))
+    return out
+
+
+HELPERS = _helpers()
+
+
+def test_the_aligned_helpers_are_found():
+    assert sorted(k[0] for k in HELPERS) == sorted(
+        ["tmem_alloc", "tmem_dealloc", "tmem_alloc_pair", "tmem_dealloc_pair", "cluster_sync", "conv_sync",
+         "o_epi_sync", "o_epi_sync_all", "o_epi_sync_and", "o_epi_sync_and_all"])
+
+
+@pytest.mark.parametrize("name,body", HELPERS, ids=[k[0] for k in HELPERS])
+def test_aligned_helpers_converge_the_warp_first(name, body):
+    first = body.find("__syncwarp()")
+    assert 0 <= first < body.index("asm"), name
+
+
+def test_product_tiles_converge_the_warp_before_they_read_tmem():
+    # one lane hands each box of 32 columns to a bulk store and is back at the next box's load
+    text = _code(os.path.join(CSRC, "k_dot.cu"))
+    loads = list(re.finditer(r"RESS_TMEM_LD32", text))
+    assert len(loads) == 2
+    for m in loads:
+        assert text[:m.start()].rstrip().endswith("__syncwarp();")
