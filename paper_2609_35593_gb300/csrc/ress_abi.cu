@@ -76,6 +76,7 @@ int check_ws(const ress::Shape& s, void* ws, size_t ws_bytes, ress_ws_layout* L)
 }
 
 int cuda_fail(cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here: a later call's cudaGetLastError must not find it again
   return fail(RESS_ECUDA, "%s: %s", where, cudaGetErrorString(e));
 }
 
