@@ -70,6 +70,12 @@ constexpr uint32_t kTileBytes = 64 * 128;    // one 64 x 64 bf16 tile
 // and its row sum accumulate in fp32, so p <= 2^20 over at most 2^18 keys stays far from
 // overflow; a stale max changes no result, the scale cancels in O / l.
 constexpr float kLazyThreshold = 20.0f;
+// Lowest reference maximum of a share of an item (log2 units).  A share may hold nothing but keys
+// that the caller masks with a huge negative score (or -inf).  Against a maximum of that size
+// the rounding of s - m alone exceeds 2^7 and the exponentials are 0 or infinite; the share's
+// weight 2^(m_s - m) is 0, and 0 * inf would make the row NaN.  Above -2^31 that rounding is at
+// most 2^6, so the exponentials stay finite; below it they are 0 against -2^31.
+constexpr float kMinRef = -2147483648.0f;
 
 struct TileInfo {
   int j, mask, flags, item;
@@ -614,6 +620,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2)
             if (m_use == -INFINITY) {
               // first kept tile of this row: O row is still zero
               m_use = row_max(x) * kScale;
+              if (kSplit) m_use = fmaxf(m_use, kMinRef);
               exps(x, m_use, w);
             } else {
               // the exponentials against the current reference run alongside the maximum;
