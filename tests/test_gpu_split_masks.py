@@ -10,6 +10,7 @@ import synth
 
 torch = pytest.importorskip("torch")
 import gpu_harness as G  # noqa: E402
+from attention64 import errors  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -25,20 +26,5 @@ def test_masked_keys(N, H, ns, lo, hi, value):
     masked = slice(64 * int(lo * nb), N if hi == 1.0 else 64 * int(hi * nb))
     inp["K"][masked, :, 63] = synth.bf16_bits(np.float32([value]))
     layer = G.Layer(inp, ns, [7] * H, 0).run_forward()  # fewer blocks than stay unmasked
-    rp, ci = layer.csr()
-    err = size = worst = 0.0
-    for h in range(H):
-        keep = np.zeros((layer.nq, nb), bool)
-        for i in range(layer.nq):
-            at = h * layer.nq + i
-            keep[i, ci[rp[at]:rp[at + 1]]] = True
-        token = torch.arange(N, device="cuda") // 64
-        keep = torch.from_numpy(keep).cuda()[token][:, token]
-        q, k, v = (x[:, h].double() for x in (layer.Q, layer.K, layer.V))
-        s = (q[:, :63] @ k[:, :63].T + k[:, 63]) / 8.0
-        want = torch.softmax(s.masked_fill(~keep, -float("inf")), dim=1) @ v
-        assert bool(torch.isfinite(want).all())  # every row keeps keys that are not masked
-        diff = (layer.buf.O[:, h].double() - want).abs()
-        worst = max(worst, float((diff - 2.0 ** -8 * want.abs()).max()))
-        err, size = err + float(diff.sum()), size + float(want.abs().sum())
-    assert worst <= G.ATT_MAX_ABS and err <= G.ATT_MEAN_REL * size, (worst, err / size)
+    worst, mean = errors(layer)  # (every row keeps keys that are not masked)
+    assert worst <= G.ATT_MAX_ABS and mean <= G.ATT_MEAN_REL, (worst, mean)
