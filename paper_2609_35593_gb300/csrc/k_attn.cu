@@ -841,9 +841,9 @@ int attn_num_pairs(const Shape& s) { return (s.nb + 1) / 2; }
 // shortest, if it is at least four tiles shorter than whole items.  Only the forward on the
 // 64-token grid, whose output is not tied bit for bit to ress_sparse_attn's (a share has its own
 // reference maxima).  The whole layer with 1 / 2 / 3 / 4 CTAs for every item: 2 views (88 items)
-// 89.8 / 85.7 / 85.3 / 100.8 us; 5,003 tokens x 3 heads (120 items, dense ones of 79 tiles) 106.7 /
-// 95.6 / 104.5 / 108.9, 90.6 with 4 for the dense ones and 2 for the others; 8 views (1,376 items) 309.9 and, with two,
-// 391.5: what does not fit into one wave loses.
+// 83.3 / 79.6 / 78.9 / 94.7 us; 5,003 tokens x 3 heads (120 items, dense ones of 79 tiles) 98.8 /
+// 87.3 / 96.1 / 100.5, 81.6 with 4 for the dense ones and 2 for the others.  What does not fit into
+// one wave loses: 8 views (1,376 items) with two CTAs each took a quarter longer.
 AttnSplit attn_split(const Shape& s, const int32_t* c_h) {
   AttnSplit best{1, 1};
   if (s.qb != kBlock) return best;

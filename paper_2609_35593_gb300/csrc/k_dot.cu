@@ -41,10 +41,10 @@
 // stores every box twice takes 42 us instead of 28, one with a sixth of the MMAs 27).  Kernel times
 // at 32 views (576 tiles): logits 14.7 -> 13.5 us, drift norms 14.9 -> 13.2, gains 14.9 -> 12.3
 // against k_dot; at 100 views (4624 tiles) 98.8 -> 67.9, 94.5 -> 67.9 and 96 -> 64.6; all of a
-// selection at 64 views (1936 tiles, six products) 1830 -> 1752 us.  Up to
-// two tiles per SM k_dot is the better one: the layer at 8 views (64 tiles) takes 301 us with it
-// and 306 with k_dot_run, whose CTA needs more of the SM before it can start beside the kernel
-// ahead of it; at 288 tiles (32 views, 128-token query blocks) they are equal, 1042 us.
+// selection at 64 views (1936 tiles, six products) 1815 -> 1752 us.  Up to
+// two tiles per SM k_dot is the better one: the layer at 8 views (64 tiles, 75% sparsity) takes 292
+// us with it and 303 with k_dot_run, whose CTA needs more of the SM before it can start beside the
+// kernel ahead of it; at 288 tiles (32 views, 128-token query blocks) they are equal, 1040 us.
 // Every mbarrier wait is bounded; a wait that gives up records RESS_ETIMEOUT, lets copies and
 // MMAs already issued finish (again bounded), frees TMEM and returns.
 

@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kOThreads, 1)
     for (int k = 0; k < nunits && !failed; ++k) {
       const OUnit t = unit_of_pair<MODE>(p, k);
       // the stripe of the pair's next unit into L2 while this one runs (by the pair that takes
-      // the stripe's first channels): 69.4 -> 67.4 us at 43,968 tokens
+      // the stripe's first channels): 69.4 -> 67.4 us at 43,968 tokens, warm inputs
       const OUnit t2 = unit_of_pair<MODE>(p, min(k + 1, nunits - 1));
       const bool ahead = MODE == kResidual && k + 1 < nunits && t2.col == 0;
       for (int ks = 0; ks < ksteps; ++ks, ++it) {
@@ -504,7 +504,7 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   const int tiles = p.mtiles * p.ntiles, slots = max(1, sm_count_of_device() / 2);
   // Tiles past the last whole wave of pairs run as 2 or 4 units of fewer channels each where
   // those fit into one wave (43,968 tokens and d_model 1024: 688 tiles on 76 pairs are nine
-  // waves and four tiles: 68.3 us with a tenth wave, 67.7 split).
+  // waves and four tiles: 68.3 us with a tenth wave, 67.7 split, warm inputs).
   p.whole = tiles;
   p.parts = 1;
   const int left = tiles % slots;
@@ -517,9 +517,10 @@ cudaError_t launch_oproj_impl(const OProjArgs& a, cudaStream_t st) {
   // cost of a tile is its K / 64 steps and an epilogue of about two; starting and ending a CTA is
   // about eight, once for persistent pairs and for every wave of clusters.  A GPC rarely has room
   // for as many clusters of 8 CTAs as its SMs would allow, so those are counted with one in eight
-  // less.  (8 views, 16 heads: 47.6 us with a pair per stripe, 50.4 in clusters of two, 44.3 of
-  // four; 16 views 94.7, 75.3 and 87.4.  84,608 tokens, 8 heads: 71.3 us with persistent pairs, 83.9
-  // with a CTA pair launched per stripe, 98.0 in clusters of two; 4 heads 25.6 and 39.2.)
+  // less.  (16 heads, L2 flushed, persistent pairs / clusters of two / of four: 8 views 54.0 / 57.0 /
+  // 49.9 us, 12 views 58.0 / 59.4 / 78.5, 16 views 103 / 84.6 / 95.9, 24 views 106 / 112 / 139, 32
+  // views 152 / 138 / 183, 100 views 376 / 391 / 528.  84,608 tokens, 8 heads: 71.3 us with persistent
+  // pairs, 83.9 with a pair launched per stripe.)
   p.group = 1;
   if (MODE == kDrift) {
     int64_t best = INT64_MAX;

@@ -277,10 +277,10 @@ __device__ __forceinline__ float sqrt_approx(float x) {
   return y;
 }
 
-// a / b for b in [2^-54, 2^4] (here a product of factors clamped at eps = 1e-4): one SFU
-// reciprocal and a multiplication.  __fdividef gives the same bits there (compared on 1e9
-// random pairs, denormal numerators included) but spends further instructions on
-// denominators outside that range.
+// a / b for b in [2^-54, 2^4] (here a product of factors clamped at eps = 1e-4), in the form the
+// PTX manual gives for div.approx: a times the approximate reciprocal of b.  Same bits as
+// __fdividef there (compared on 1e9 random pairs, denormal numerators included); selection at 64
+// views 1752 us against 1759 with __fdividef, the 32-view layer 1329 and 1330.
 __device__ __forceinline__ float div_fast(float a, float b) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));

@@ -406,10 +406,10 @@ int yagg_ranges(const Shape& s) {
 
 // A CTA per range where that takes at least 6 chunks off a CTA's chain of them: handing partial
 // sums over through scratch (stores, fence, counter, loads) costs about as much as 6 chunks.
-// Layer with a CTA per range against all ranges in one CTA, three ranges, 16 heads: 3 chunks
-// (8 views) 222.5 and 214.4 us, 5 (12 views) 318.2 and 311.9, 6 (16) 448.6 and 445.7, 128-token
-// query blocks 6 (16) 378.8 and 372.5, 9 (24) 684.0 and 684.5, 11 (32) 1036.4 and 1039.4.  The
-// 8-view kernel itself takes 14.1 us instead of 20.0.
+// Layer of 16 heads at 90% sparsity with a CTA per range against all ranges in one CTA, three
+// ranges: 3 chunks (8 views) 226.9 and 218.8 us, 5 (12 views) 320.3 and 313.8, 6 (16) 452.2 and
+// 449.7, 128-token query blocks 6 (16) 381.2 and 375.1, 9 (24) 688.0 and 689.1, 11 (32) 1039.7 and
+// 1042.8.  At 75% sparsity the 8-view layer takes 301 and 292.6; its kernel 20.0 and 14.1.
 int yagg_parts(const Shape& s) {
   const int nchunks = (s.nb + kYChunk - 1) / kYChunk, k = yagg_ranges(s);
   return nchunks - (nchunks + k - 1) / k >= 6 ? k : 1;

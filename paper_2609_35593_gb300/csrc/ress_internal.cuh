@@ -156,8 +156,8 @@ void note_launch();
 // Launches a kernel that may start before the kernel ahead of it in the stream has finished
 // (programmatic dependent launch), so that its launch and its set-up (barriers, TMEM,
 // constants in shared memory) overlap the other's last CTAs; see ptx::pdl_wait for what the
-// kernel has to do.  One forward is 15 launches: 2 views 122 -> 91 us, 8 views 337 -> 306 us,
-// 32 views 1384 -> 1357 us.  overlap = false: an ordinary launch of the same kernel.
+// kernel has to do.  One forward is 15 launches: 109.6 us without and 79.0 with it at 2 views, 322
+// and 292 at 8, 1361 and 1329 at 32.  overlap = false: an ordinary launch of the same kernel.
 template <typename... P, typename... A>
 cudaError_t launch_with(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                         bool overlap, dim3 cluster, const A&... args) {

@@ -31,8 +31,8 @@ __device__ __forceinline__ bool elect_one() {
 // the stream may start its CTAs once every CTA of this one has triggered or ended.  It stands
 // after the wait and late in each kernel, when the CTA has only its last stage left: a trigger
 // at the top lets several later kernels queue up on the SMs, whose CTAs then sit unevenly
-// (8-view layer: 337 us without overlap, 343 with the trigger at the top, 312 right after the
-// wait, 306 late), and it could let a later kernel's CTA take TMEM that a CTA of an earlier one
+// (8-view layer of that time: 337 us without overlap, 343 with the trigger at the top, 312 right
+// after the wait, 306 late), and it could let a later kernel's CTA take TMEM that a CTA of an earlier one
 // has yet to allocate.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
